@@ -117,6 +117,22 @@ struct CloverAoS16 {
     const uint4* p;  // [V][9]: the 72 packed reals as halves
 };
 
+// 4^4 blocks: the same words with all of a block's sites side by side, [V / 256][word][256], so that
+// the 16-byte loads of consecutive sites are contiguous and every word is at a constant offset from
+// the block's base address
+struct LinksB {
+    const float4* p;  // [NB][4][5][256]
+};
+struct CloverB {
+    const float4* p;  // [NB][18][256]
+};
+struct LinksB16 {
+    const uint4* p;  // [NB][4][3][256]
+};
+struct CloverB16 {
+    const uint4* p;  // [NB][2][5][256]: each hermitian block's 36 halves padded to 40
+};
+
 struct Geom {
     int V;       // fine sites
     int Vb;      // sites per block

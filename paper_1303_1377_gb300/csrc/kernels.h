@@ -25,6 +25,15 @@ struct FineOpAoS16 {
     CloverAoS16 clov, clovinv;
 };
 
+struct FineOpB {  // 4^4 blocks
+    LinksB U;
+    CloverB clov, clovinv;
+};
+struct FineOpB16 {
+    LinksB16 U;
+    CloverB16 clov, clovinv;
+};
+
 // coarse stencil in storage type S (float, double or __half2 packed as cplx<half>)
 template <typename S>
 struct CoarseOp {
@@ -48,17 +57,22 @@ int launch_sap_colour_aos(const Geom& g, const FineOpAoS& op, const cplx<float>*
 bool sap_aos_supported(const Geom& g, int nrhs);
 int launch_sap_colour_aos16(const Geom& g, const FineOpAoS16& op, const cplx<float>* b, cplx<float>* z, int colour, int nrhs,
                             int mr_steps, cudaStream_t st);
-// FP32 [comp][V] -> FP16 per-site copies (links [V][4][3] uint4, site term [V][9] uint4)
-int links_to_aos16(const cplx<float>* U, uint4* out, int V, cudaStream_t st);
-int clover_to_aos16(const float* cl, uint4* out, int V, cudaStream_t st);
+// FP32 [comp][V] -> FP16 per-site copies (links [V][4][3] uint4, site term [V][9] uint4); blocked: the
+// same words per 4^4 block, [V / 256][word][256]
+int links_to_aos16(const cplx<float>* U, uint4* out, int V, bool blocked, cudaStream_t st);
+int clover_to_aos16(const float* cl, uint4* out, int V, bool blocked, cudaStream_t st);
 // [comp][V] -> per-site copies (links: 4 x 9 complex -> [V][4][5] float4; site term: 72 -> [V][18] float4)
-int links_to_aos(const cplx<float>* U, float4* out, int V, cudaStream_t st);
-int clover_to_aos(const float* cl, float4* out, int V, cudaStream_t st);
+int links_to_aos(const cplx<float>* U, float4* out, int V, bool blocked, cudaStream_t st);
+int clover_to_aos(const float* cl, float4* out, int V, bool blocked, cudaStream_t st);
 int upload_gamma_products(const double* gg);
 int launch_dslash_dw(const Geom& g, const float4* U, const float2* clov, const cplx<float>* in, void* out, bool out_dw, int nrhs,
                      cudaStream_t st);
 int launch_to_dw(const double* in, float2* out, size_t n, cudaStream_t st);
 int launch_clover(const Geom& g, const cplx<double>* U, double m0, double csw, double* clov, double* clovinv, cudaStream_t st);
+
+// ---- sap44.cu: FP32 SAP sweep on 4^4 blocks (FineOpB, FineOpB16)
+template <typename OpT>
+int launch_sap44(const Geom& g, const OpT& op, const cplx<float>* b, cplx<float>* z, int colour, int nrhs, int mr_steps, cudaStream_t st);
 
 // ---- transfer.cu (P, P^H, Gram-Schmidt, D_c assembly)
 template <typename T, typename Tp>

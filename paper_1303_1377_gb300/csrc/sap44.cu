@@ -1,0 +1,294 @@
+// Red-black SAP block solver (Sec. 2.3, local odd-even MR of Sec. 6) on 4^4 blocks in FP32 arithmetic.
+//
+// A CTA of 128 threads owns one block of the colour and two right-hand sides; each thread owns one even
+// and one odd site and computes both right-hand sides in packed FP32 instructions (f32x2.cuh), so a link
+// or site-term entry is loaded and converted once for two right-hand sides and a multiply-add issues
+// once for two.  x_o stays in registers (255 a thread, two CTAs per SM); the even work vector and rho
+// take 49 KB of shared memory, which leaves the rest of the SM's 256 KB to L1 for the links and site
+// terms that every MR step reads again.
+//
+// What bounds it: the packed multiply-adds (two cycles each) hold the FMA pipe about 60% busy in the MR
+// steps; the residual at the start waits on its neighbours' spinors.  12 fields on 24^4, one colour,
+// FP16 operator: 740 us (29 TFLOP/s) against 1347 us for one right-hand side per thread, four per CTA
+// (512 threads, 128 registers); FP32 operator 740 against 1399 us; one field 151 against 212 us.  Tried
+// and slower (same case): four right-hand sides per CTA 778 us, six 806 us; x_o in shared memory
+// (+12%); the links in shared memory as FP32 (+5%); two threads per site split by spin 781 us; own z
+// and the faces staged through shared memory (+15%).
+#include <type_traits>
+
+#include "block44.cuh"
+#include "f32x2.cuh"
+#include "kernels.h"
+
+namespace ddamg {
+
+// ---- operator copies of the 4^4 blocks (common.cuh): all words of a block sit together, [word][site]
+// W = U_mu at local site l of block c; on = false: zero, nothing is read
+__device__ __forceinline__ void load_link44(cplx<float> (&W)[9], const LinksB& U, int c, int mu, int l, bool on = true) {
+    const float4* q = U.p + (size_t)c * (20 * 256) + mu * (5 * 256) + l;
+    const float4 zero = make_float4(0.f, 0.f, 0.f, 0.f);
+    float4 a = zero, b = zero, d = zero, e = zero, f = zero;
+    if (on) a = __ldg(q), b = __ldg(q + 256), d = __ldg(q + 512), e = __ldg(q + 768), f = __ldg(q + 1024);
+    W[0] = mk(a.x, a.y), W[1] = mk(a.z, a.w), W[2] = mk(b.x, b.y), W[3] = mk(b.z, b.w), W[4] = mk(d.x, d.y);
+    W[5] = mk(d.z, d.w), W[6] = mk(e.x, e.y), W[7] = mk(e.z, e.w), W[8] = mk(f.x, f.y);
+}
+__device__ __forceinline__ void load_link44(cplx<float> (&W)[9], const LinksB16& U, int c, int mu, int l, bool on = true) {
+    const uint4* q = U.p + (size_t)c * (12 * 256) + mu * (3 * 256) + l;
+    uint4 a = make_uint4(0u, 0u, 0u, 0u), b = a;
+    unsigned d = 0u;
+    if (on) a = __ldg(q), b = __ldg(q + 256), d = __ldg(&(q + 512)->x);
+    const unsigned w[9] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w, d};
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const float2 f = h2f(w[k]);
+        W[k] = mk(f.x, f.y);
+    }
+}
+// y = (block h of the site term) x, h = 0, 1
+template <int HB>
+__device__ __forceinline__ void herm44(const CloverB& cl, int c, int l, const c2 (&x)[6], c2 (&y)[6]) {
+    const float4* q = cl.p + (size_t)c * (18 * 256) + HB * (9 * 256) + l;
+    float w[36];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const float4 v = __ldg(q + k * 256);
+        w[4 * k] = v.x, w[4 * k + 1] = v.y, w[4 * k + 2] = v.z, w[4 * k + 3] = v.w;
+    }
+    herm6_apply2([&](int j) { return w[j]; }, x, y);
+}
+template <int HB>
+__device__ __forceinline__ void herm44(const CloverB16& cl, int c, int l, const c2 (&x)[6], c2 (&y)[6]) {
+    const uint4* q = cl.p + (size_t)c * (10 * 256) + HB * (5 * 256) + l;
+    unsigned w[20];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const uint4 v = __ldg(q + k * 256);
+        w[4 * k] = v.x, w[4 * k + 1] = v.y, w[4 * k + 2] = v.z, w[4 * k + 3] = v.w;
+    }
+    herm6_apply2(
+        [&](int j) {
+            const float2 f = h2f(w[j / 2]);
+            return (j & 1) ? f.y : f.x;
+        },
+        x, y);
+}
+
+// ---- hops
+// in-block hops in direction MU of local site (lexicographic index L, local index l) of block c; sm
+// holds the field on the other parity (rank order), nb0 = local index of rank 0 of that parity.  A
+// neighbour outside the block is replaced by the one on the other side with a zero link: a quarter of
+// the lanes would idle in a branch anyway, and without branches the loads of the next hops are issued
+// while the current one computes (one MR step of 12 fields on 24^4: 121 us with branches, 96 us without).
+template <int MU, typename UT>
+__device__ __forceinline__ void hop_pair44(const UT& U, const float4* sm, int L, int nb0, int c, int l, c2 (&acc)[12]) {
+    constexpr int SH = 2 * (3 - MU), S = 1 << SH;
+    const int y = (L >> SH) & 3;
+    const bool f = y < 3, b = y > 0;
+    const int nf = (f ? L + S : L - S) >> 1, nb = (b ? L - S : L + S) >> 1;
+    cplx<float> Wf[9], Wb[9];
+    load_link44(Wf, U, c, MU, l, f);
+    load_link44(Wb, U, c, MU, nb0 + nb, b);
+    hop_acc2<MU, true>(acc, [&](int k) { return c2_of(sm[k * 128 + nf]); }, Wf);
+    hop_acc2<MU, false>(acc, [&](int k) { return c2_of(sm[k * 128 + nb]); }, Wb);
+}
+template <typename UT>
+__device__ __forceinline__ void hops44(const UT& U, const float4* sm, int L, int nb0, int c, int l, c2 (&acc)[12]) {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = c2zero();
+    hop_pair44<0>(U, sm, L, nb0, c, l, acc);
+    hop_pair44<1>(U, sm, L, nb0, c, l, acc);
+    hop_pair44<2>(U, sm, L, nb0, c, l, acc);
+    hop_pair44<3>(U, sm, L, nb0, c, l, acc);
+}
+// both hops of D in direction MU with the field read from global memory
+template <int MU, typename UT>
+__device__ __forceinline__ void hop_pair44_global(const UT& U, const cplx<float>* z0, const cplx<float>* z1, int V, int L, int p, int c,
+                                                  int bf, int bb, c2 (&acc)[12]) {
+    cplx<float> W[9];
+    const int f = nbr44<MU, true>(L, p, c, bf), b = nbr44<MU, false>(L, p, c, bb);
+    load_link44(W, U, c, MU, (p << 7) | (L >> 1));
+    hop_acc2<MU, true>(acc, [&](int k) { return c2pair(z0[(size_t)k * V + f], z1[(size_t)k * V + f]); }, W);
+    load_link44(W, U, b >> 8, MU, b & 255);
+    hop_acc2<MU, false>(acc, [&](int k) { return c2pair(z0[(size_t)k * V + b], z1[(size_t)k * V + b]); }, W);
+}
+
+template <typename OpT>
+__global__ void __launch_bounds__(128, 2)
+    sap44_kernel(Geom g, OpT op, const cplx<float>* __restrict__ bsrc, cplx<float>* z, int colour, int nrhs, int mr_steps, int npairs) {
+    constexpr int H = 128;
+    extern __shared__ float4 smem44[];
+    const int t = threadIdx.x, r0 = 2 * (blockIdx.x % npairs);
+    const bool two = r0 + 1 < nrhs;  // an odd batch computes its last right-hand side twice and stores it once
+    float4* SE = smem44;                                         // [12][H] even work vector
+    float4* SO = SE + 12 * H;                                    // [12][H] r_o, then rho, then x_o
+    float2* red = reinterpret_cast<float2*>(smem44 + 24 * H);    // [4 warps][3]
+    const int V = g.V, c = colour * (g.NB / 2) + blockIdx.x / npairs;
+    const cplx<float>* b0 = bsrc + (size_t)r0 * 12 * V;
+    const cplx<float>* b1 = b0 + (two ? (size_t)12 * V : 0);
+    cplx<float>* z0 = z + (size_t)r0 * 12 * V;
+    cplx<float>* z1 = z0 + (two ? (size_t)12 * V : 0);
+    const int ie = c * 256 + t, io = ie + H;
+    // z += d at component k0 .. k0 + n - 1 of site i: all loads before the first store (a store ends
+    // what the compiler can prove about the other components, so a plain loop waits for each load)
+    auto add_z = [&](int k0, int i, const c2* d, auto n) {
+        constexpr int N = decltype(n)::value;
+        cplx<float> u[N], v[N];
+#pragma unroll
+        for (int a = 0; a < N; ++a) u[a] = z0[(size_t)(k0 + a) * V + i], v[a] = z1[(size_t)(k0 + a) * V + i];
+#pragma unroll
+        for (int a = 0; a < N; ++a) {
+            z0[(size_t)(k0 + a) * V + i] = u[a] + mk(d[a].re.x, d[a].im.x);
+            if (two) z1[(size_t)(k0 + a) * V + i] = v[a] + mk(d[a].re.y, d[a].im.y);
+        }
+    };
+    using I6 = std::integral_constant<int, 6>;
+    using I12 = std::integral_constant<int, 12>;
+    // residual r = b - D z; even sites: SE = A_ee^{-1} r_e, odd sites: SO = r_o
+#pragma unroll 1
+    for (int p = 0; p < 2; ++p) {
+        const int l = p * H + t, i = c * 256 + l, L = lex44_of_local(l);
+        int bn[8];
+#pragma unroll
+        for (int d = 0; d < 8; ++d) bn[d] = __ldg(g.bnbr + d * g.NB + c);
+        c2 acc[12];
+#pragma unroll
+        for (int k = 0; k < 12; ++k) acc[k] = c2zero();
+        hop_pair44_global<0>(op.U, z0, z1, V, L, p, c, bn[0], bn[1], acc);
+        hop_pair44_global<1>(op.U, z0, z1, V, L, p, c, bn[2], bn[3], acc);
+        hop_pair44_global<2>(op.U, z0, z1, V, L, p, c, bn[4], bn[5], acc);
+        hop_pair44_global<3>(op.U, z0, z1, V, L, p, c, bn[6], bn[7], acc);
+        c2 x[6], y[6];
+        auto half = [&](auto hb) {
+            constexpr int HB = decltype(hb)::value;
+#pragma unroll
+            for (int a = 0; a < 6; ++a) x[a] = c2pair(z0[(size_t)(HB * 6 + a) * V + i], z1[(size_t)(HB * 6 + a) * V + i]);
+            herm44<HB>(op.clov, c, l, x, y);
+#pragma unroll
+            for (int a = 0; a < 6; ++a) {
+                const size_t o = (size_t)(HB * 6 + a) * V + i;
+                x[a] = c2pair(b0[o], b1[o]) - c2axpy(y[a], -0.5f, acc[HB * 6 + a]);
+            }
+            if (p == 0) {
+                herm44<HB>(op.clovinv, c, l, x, y);
+#pragma unroll
+                for (int a = 0; a < 6; ++a) SE[(HB * 6 + a) * H + t] = c2_f4(y[a]);
+            } else {
+#pragma unroll
+                for (int a = 0; a < 6; ++a) SO[(HB * 6 + a) * H + t] = c2_f4(x[a]);
+            }
+        };
+        half(std::integral_constant<int, 0>());
+        half(std::integral_constant<int, 1>());
+    }
+    __syncthreads();  // every read of z in this block is done: z may be updated from here on
+    c2 xo[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) xo[k] = c2_of(SE[k * H + t]);
+    add_z(0, ie, xo, I12());  // the part A_ee^{-1} r_e of x_e, which does not depend on x_o
+#pragma unroll
+    for (int k = 0; k < 12; ++k) xo[k] = c2zero();
+    const int Le = lex44_of_local(t), Lo = lex44_of_local(H + t);
+    // pass 0 forms rho = r_o - D_oe A_ee^{-1} r_e; passes 1 .. mr_steps are the MR steps on
+    // S = A_oo - D_oe A_ee^{-1} D_eo; the even half of the last pass is the back-substitution
+#pragma unroll 1
+    for (int it = 0; it <= mr_steps; ++it) {
+        {
+            c2 sr[12];
+            hops44(op.U, SE, Lo, 0, c, H + t, sr);
+            if (it == 0) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) SO[k * H + t] = c2_f4(c2axpy(c2_of(SO[k * H + t]), 0.5f, sr[k]));
+            } else {
+                float2 nr = make_float2(0.f, 0.f), ni = nr, dd = nr;
+                auto half = [&](auto hb) {
+                    constexpr int HB = decltype(hb)::value;
+                    c2 rho[6], y[6];
+#pragma unroll
+                    for (int a = 0; a < 6; ++a) rho[a] = c2_of(SO[(HB * 6 + a) * H + t]);
+                    herm44<HB>(op.clov, c, H + t, rho, y);
+#pragma unroll
+                    for (int a = 0; a < 6; ++a) {
+                        const c2 s = c2axpy(y[a], 0.5f, sr[HB * 6 + a]);
+                        sr[HB * 6 + a] = s;
+                        nr = f2fma(s.re, rho[a].re, nr), nr = f2fma(s.im, rho[a].im, nr);
+                        ni = f2fma(s.re, rho[a].im, ni), ni = f2fma(f2neg(s.im), rho[a].re, ni);
+                        dd = f2fma(s.re, s.re, dd), dd = f2fma(s.im, s.im, dd);
+                    }
+                };
+                half(std::integral_constant<int, 0>());
+                half(std::integral_constant<int, 1>());
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1) {
+                    nr.x += __shfl_xor_sync(0xffffffffu, nr.x, o), nr.y += __shfl_xor_sync(0xffffffffu, nr.y, o);
+                    ni.x += __shfl_xor_sync(0xffffffffu, ni.x, o), ni.y += __shfl_xor_sync(0xffffffffu, ni.y, o);
+                    dd.x += __shfl_xor_sync(0xffffffffu, dd.x, o), dd.y += __shfl_xor_sync(0xffffffffu, dd.y, o);
+                }
+                if ((t & 31) == 0) red[3 * (t >> 5)] = nr, red[3 * (t >> 5) + 1] = ni, red[3 * (t >> 5) + 2] = dd;
+                __syncthreads();
+                nr = f2add(f2add(red[0], red[3]), f2add(red[6], red[9]));
+                ni = f2add(f2add(red[1], red[4]), f2add(red[7], red[10]));
+                dd = f2add(f2add(red[2], red[5]), f2add(red[8], red[11]));
+                const bool ok0 = dd.x > tiny_normal<float>(), ok1 = dd.y > tiny_normal<float>();
+                const float2 ar = make_float2(ok0 ? nr.x / dd.x : 0.f, ok1 ? nr.y / dd.y : 0.f);
+                const float2 ai = make_float2(ok0 ? ni.x / dd.x : 0.f, ok1 ? ni.y / dd.y : 0.f);
+                const float2 mr = f2neg(ar), mi = f2neg(ai);
+                const bool last = it == mr_steps;
+#pragma unroll
+                for (int k = 0; k < 12; ++k) {  // x_o += alpha rho, rho -= alpha S rho
+                    const c2 rho = c2_of(SO[k * H + t]);
+                    xo[k].re = f2fma(mi, rho.im, f2fma(ar, rho.re, xo[k].re));
+                    xo[k].im = f2fma(ai, rho.re, f2fma(ar, rho.im, xo[k].im));
+                    c2 nw;
+                    nw.re = f2fma(ai, sr[k].im, f2fma(mr, sr[k].re, rho.re));
+                    nw.im = f2fma(mi, sr[k].re, f2fma(mr, sr[k].im, rho.im));
+                    if (!last) SO[k * H + t] = c2_f4(nw);
+                }
+            }
+            if (it == mr_steps) {
+#pragma unroll
+                for (int k = 0; k < 12; ++k) SO[k * H + t] = c2_f4(xo[k]);
+            }
+        }
+        __syncthreads();
+        {
+            c2 hs[12];
+            hops44(op.U, SO, Le, H, c, t, hs);
+            const bool last = it == mr_steps;
+            auto half = [&](auto hb) {
+                constexpr int HB = decltype(hb)::value;
+                c2 x[6], y[6];
+#pragma unroll
+                for (int a = 0; a < 6; ++a) x[a] = c2scale(last ? 0.5f : -0.5f, hs[HB * 6 + a]);
+                herm44<HB>(op.clovinv, c, t, x, y);
+                if (last) add_z(HB * 6, ie, y, I6());
+                else {
+#pragma unroll
+                    for (int a = 0; a < 6; ++a) SE[(HB * 6 + a) * H + t] = c2_f4(y[a]);
+                }
+            };
+            half(std::integral_constant<int, 0>());
+            half(std::integral_constant<int, 1>());
+        }
+        __syncthreads();
+    }
+    add_z(0, io, xo, I12());
+}
+
+template <typename OpT>
+int launch_sap44(const Geom& g, const OpT& op, const cplx<float>* b, cplx<float>* z, int colour, int nrhs, int mr_steps, cudaStream_t st) {
+    const size_t smem = 24 * 128 * sizeof(float4) + 12 * sizeof(float2);
+    // set once per kernel instance (a function-local static initialiser is thread safe)
+    static const bool attr = [] {
+        cudaFuncSetAttribute(sap44_kernel<OpT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
+        return true;
+    }();
+    (void)attr;
+    const int npairs = (nrhs + 1) / 2;
+    sap44_kernel<OpT><<<(unsigned)(g.NB / 2) * (unsigned)npairs, 128, smem, st>>>(g, op, b, z, colour, nrhs, mr_steps, npairs);
+    DD_CHECK_LAUNCH();
+    return 0;
+}
+template int launch_sap44(const Geom&, const FineOpB&, const cplx<float>*, cplx<float>*, int, int, int, cudaStream_t);
+template int launch_sap44(const Geom&, const FineOpB16&, const cplx<float>*, cplx<float>*, int, int, int, cudaStream_t);
+
+}  // namespace ddamg

@@ -588,8 +588,18 @@ static int sap(ddamg_handle* h, const cplx<T>* b, cplx<T>* z, int nrhs, int nu) 
             if constexpr (std::is_same<T, float>::value) {
                 if (f16) {
                     // half-precision V-cycle: links and site terms of the smoother stored in FP16
+                    if (h->g.blk44) {
+                        const FineOpB16 op{LinksB16{h->Uaos16}, CloverB16{h->clov_aos16}, CloverB16{h->clovinv_aos16}};
+                        DD_TRY(launch_sap44(h->g, op, b, z, colour, nrhs, h->p.mr_steps, h->stream));
+                        continue;
+                    }
                     const FineOpAoS16 op{LinksAoS16{h->Uaos16}, CloverAoS16{h->clov_aos16}, CloverAoS16{h->clovinv_aos16}};
                     DD_TRY(launch_sap_colour_aos16(h->g, op, b, z, colour, nrhs, h->p.mr_steps, h->stream));
+                    continue;
+                }
+                if (h->g.blk44) {
+                    const FineOpB op{LinksB{h->Uaos}, CloverB{h->clov_aos}, CloverB{h->clovinv_aos}};
+                    DD_TRY(launch_sap44(h->g, op, b, z, colour, nrhs, h->p.mr_steps, h->stream));
                     continue;
                 }
                 if (sap_aos_supported(h->g, nrhs)) {
@@ -1609,8 +1619,9 @@ static int create(const ddamg_lattice* lat, const double* U, double m0, double c
         if ((rc = dalloc_n(&h->d_tc_err, 1))) return fail(rc);
         if (cudaMemset(h->d_tc_err, 0, sizeof(int)) != cudaSuccess) return fail(DDAMG_ERR_CUDA);
         h->tc = CoarseTC{h->Bh, h->Dh, h->d_bnbr, h->NB, (int)nc, Mt, Kta, Kth, Ktd, h->d_tc_err};
+        const size_t cw16 = h->g.blk44 ? 10 : 9;  // 16-byte words of a site term (clover_to_aos16)
         if (p.smoother_fp16 &&
-            ((rc = dalloc_n(&h->Uaos16, V * 12)) || (rc = dalloc_n(&h->clov_aos16, V * 9)) || (rc = dalloc_n(&h->clovinv_aos16, V * 9))))
+            ((rc = dalloc_n(&h->Uaos16, V * 12)) || (rc = dalloc_n(&h->clov_aos16, V * cw16)) || (rc = dalloc_n(&h->clovinv_aos16, V * cw16))))
             return fail(rc);
     } else if (h->single()) {
         if ((rc = dalloc_n(&h->P32, V * 12 * N)) || (rc = dalloc_n(&h->B32, (size_t)h->NB * 9 * nc * nc * 2)) ||
@@ -1627,13 +1638,13 @@ static int create(const ddamg_lattice* lat, const double* U, double m0, double c
             (rc = convert<float, double>(h->clov64, h->clov32, V * 72, h->stream)) ||
             (rc = convert<float, double>(h->clovinv64, h->clovinv32, V * 72, h->stream)) ||
             (rc = launch_to_dw(reinterpret_cast<const double*>(h->U64), reinterpret_cast<float2*>(h->Udw), V * 72, h->stream)) ||
-            (rc = launch_to_dw(h->clov64, h->clovdw, V * 72, h->stream)) || (rc = links_to_aos(h->U32, h->Uaos, h->V, h->stream)) ||
-            (rc = clover_to_aos(h->clov32, h->clov_aos, h->V, h->stream)) ||
-            (rc = clover_to_aos(h->clovinv32, h->clovinv_aos, h->V, h->stream)))
+            (rc = launch_to_dw(h->clov64, h->clovdw, V * 72, h->stream)) || (rc = links_to_aos(h->U32, h->Uaos, h->V, h->g.blk44, h->stream)) ||
+            (rc = clover_to_aos(h->clov32, h->clov_aos, h->V, h->g.blk44, h->stream)) ||
+            (rc = clover_to_aos(h->clovinv32, h->clovinv_aos, h->V, h->g.blk44, h->stream)))
             return fail(rc);
-        if (h->half() && h->p.smoother_fp16 && ((rc = links_to_aos16(h->U32, h->Uaos16, h->V, h->stream)) ||
-                          (rc = clover_to_aos16(h->clov32, h->clov_aos16, h->V, h->stream)) ||
-                          (rc = clover_to_aos16(h->clovinv32, h->clovinv_aos16, h->V, h->stream))))
+        if (h->half() && h->p.smoother_fp16 && ((rc = links_to_aos16(h->U32, h->Uaos16, h->V, h->g.blk44, h->stream)) ||
+                          (rc = clover_to_aos16(h->clov32, h->clov_aos16, h->V, h->g.blk44, h->stream)) ||
+                          (rc = clover_to_aos16(h->clovinv32, h->clovinv_aos16, h->V, h->g.blk44, h->stream))))
             return fail(rc);
     }
     if (cudaStreamSynchronize(h->stream) != cudaSuccess) {
@@ -2251,11 +2262,11 @@ int ddamg_set_mass(ddamg_handle* h, double m0) {
         DD_TRY((convert<float, double>(h->clov64, h->clov32, (size_t)h->V * 72, h->stream)));
         DD_TRY((convert<float, double>(h->clovinv64, h->clovinv32, (size_t)h->V * 72, h->stream)));
         DD_TRY(launch_to_dw(h->clov64, h->clovdw, (size_t)h->V * 72, h->stream));
-        DD_TRY(clover_to_aos(h->clov32, h->clov_aos, h->V, h->stream));
-        DD_TRY(clover_to_aos(h->clovinv32, h->clovinv_aos, h->V, h->stream));
+        DD_TRY(clover_to_aos(h->clov32, h->clov_aos, h->V, h->g.blk44, h->stream));
+        DD_TRY(clover_to_aos(h->clovinv32, h->clovinv_aos, h->V, h->g.blk44, h->stream));
         if (h->half() && h->p.smoother_fp16) {
-            DD_TRY(clover_to_aos16(h->clov32, h->clov_aos16, h->V, h->stream));
-            DD_TRY(clover_to_aos16(h->clovinv32, h->clovinv_aos16, h->V, h->stream));
+            DD_TRY(clover_to_aos16(h->clov32, h->clov_aos16, h->V, h->g.blk44, h->stream));
+            DD_TRY(clover_to_aos16(h->clovinv32, h->clovinv_aos16, h->V, h->g.blk44, h->stream));
         }
     }
     if (h->ready) {
