@@ -347,7 +347,8 @@ void ddamg_debug_fail_allocs(int n);
  * P_1, D_2 and its inverses are built in FP64; the level-1 and level-2 solves run in the handle's
  * V-cycle precision (FP64 on DOUBLE handles, FP32 on SINGLE and HALF handles, with FP32 copies of
  * D_1, P_1, D_2 and the inverses).  HALF handles also keep FP16 copies: the level-1 SAP reads D_1 and
- * its even inverses in FP16 (FP32 arithmetic), and the coarsest level's GMRES and ddamg_ml_apply_D2
+ * its even inverses in FP16 (the vectors enter in FP32, or as FP16 hi + lo pairs on the tensor cores,
+ * with FP32 accumulation), and the coarsest level's GMRES and ddamg_ml_apply_D2
  * apply D_2 (and its even inverses) from FP16 tensor-core fragments, with each right-hand-side entry
  * entering as an FP16 hi + lo pair so that the product is the FP16-rounded matrix times the FP32
  * vector to about 2^-22 (2 n_vec1 divisible by 8; otherwise FP32).  The third level is tied to the coarse operator it was built

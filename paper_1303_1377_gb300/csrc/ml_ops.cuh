@@ -40,6 +40,7 @@ struct MLView {
     // order), read by the fused SAP colour step only; null otherwise
     const void* B1h = nullptr;
     const void* Dinv1h = nullptr;
+    bool frag = false;  // the FP16 copies are in tensor-core fragment order (ml_sap_tc.cu)
 };
 
 template <typename T>
@@ -440,6 +441,11 @@ struct MLHostExec {
 // one SAP colour step of ml_sap as a single kernel (ml_sap.cu): FP32, blocks with as many even as
 // odd sites, at most 384 (block-half sites x components) threads and the six half-block MR vectors
 // of 12 right-hand sides within shared memory
+// the same step on tensor cores for the FP16 copies in fragment order (ml_sap_tc.cu), and their packing
+// from nblk FP64 column-major nc x nc blocks
+bool ml_sap_tc_supported(int nc, int Vb1, int Vb1e);
+int launch_ml_sap_tc(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps, cudaStream_t st);
+int pack_ml_frag(const double* in, void* out, size_t nblk, int nc, cudaStream_t st);
 bool ml_sap_fused_supported(const MLView<float>& v);
 int launch_ml_sap_fused(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps,
                         cudaStream_t st);

@@ -43,3 +43,37 @@ def test_sap_on_4x4x4x4_blocks_by_right_hand_sides(prec, tol, dims, nrhs, mr):
     ref = np.stack([sap.apply(b[r], 2) for r in range(nrhs)])
     for r in range(nrhs):
         assert np.max(np.abs(got[r] - ref[r])) < tol * np.max(np.abs(ref[r]))
+
+
+@pytest.mark.parametrize("n_vec", [8, 12, 20])
+def test_level1_sap_on_tensor_cores(n_vec):
+    """The half-precision level-1 SAP (FP16 D_1 and D_ee^{-1}, split right-hand sides) against the
+    oracle's SAP on the operator rounded as stored: a product errs by about 2^-22 (split) +
+    sqrt(9 * 2N) 2^-24 (FP32 accumulation) <= 1.4e-6 of the field maximum, and two iterations with MR(4)
+    amplify a rounding error by less than 10, so 1e-5 is asserted.  Every right-hand side is
+    independent of its group: full, partial and many-group batches agree bit for bit."""
+    from oracle.lattice import Lattice
+    from oracle.multilevel import StencilOperator, StencilSAP
+    from paper_1303_1377_gb300 import ddamg
+
+    dims, blk = (8, 8, 8, 8), (2, 2, 2, 2)
+    s, _ = _solver(dims, n_vec=n_vec, block=blk, precision=ddamg.PREC_HALF)
+    with s:
+        s.setup_from_vectors(synth.random_test_vectors(dims, n_vec, seed=31))
+        s.ml_build(synth.gaussian_coarse(256, 2 * n_vec, 3, seed=32), ddamg.ml_default_params(n_vec1=3))
+        B = s.coarse_stencil()
+        x = synth.gaussian_coarse(256, 2 * n_vec, 77, seed=33)
+        all77 = s.ml_apply_sap1(x, 2)
+        for a, b in ((0, 1), (1, 6), (6, 18)):
+            assert np.array_equal(s.ml_apply_sap1(x[a:b], 2), all77[a:b])
+
+    def r16(v):
+        return v.real.astype(np.float32).astype(np.float16) + 1j * v.imag.astype(np.float32).astype(np.float16).astype(np.float64)
+
+    op = StencilOperator(Lattice((4, 4, 4, 4)), r16(B))
+    sap = StencilSAP(op, (2, 2, 2, 2), mr_steps=4)
+    inv = r16(np.linalg.inv(B[:, 0]))
+    sap.apply_Aee_inv = lambda f: np.einsum("xij,xj->xi", inv, f)
+    for r in (0, 41):
+        ref = sap.apply(x[r], 2)
+        assert np.max(np.abs(all77[r] - ref)) < 1e-5 * np.max(np.abs(ref))
