@@ -40,7 +40,7 @@ __device__ __forceinline__ void hop_pair_nb(const UT& U, const cplx<Ts>* __restr
 template <typename T, typename Ts, bool RESID>
 __global__ void __launch_bounds__(sizeof(T) == 4 ? 384 : 128, sizeof(T) == 4 ? 2 : 1)
     dslash44_kernel(Geom g, FineOp<T> op, const int* __restrict__ blex, const cplx<Ts>* __restrict__ in, const cplx<T>* __restrict__ b,
-                    cplx<T>* __restrict__ out, int nrhs) {
+                    cplx<T>* __restrict__ out, int nrhs, const int* __restrict__ lex) {
     const int r = blockIdx.y * blockDim.y + threadIdx.y;
     const int q = blockIdx.x >> 3;
     const int l = (blockIdx.x & 7) * 32 + threadIdx.x;
@@ -64,6 +64,17 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 384 : 128, sizeof(T) == 4 ? 2
     load_spinor(x, inr, g.V, i);
     herm_apply(op.clov, g.V, i, x, y);
     cplx<T>* o = out + off;
+    if constexpr (sizeof(T) == 4 && !RESID) {
+        if (lex) {  // the caller's layout: a site's 96 bytes in 16-byte words
+            float4* w = reinterpret_cast<float4*>(o + (size_t)__ldg(lex + i) * 12);
+#pragma unroll
+            for (int k = 0; k < 12; k += 2) {
+                const cplx<T> d = y.v[k] - T(0.5) * acc.v[k], e = y.v[k + 1] - T(0.5) * acc.v[k + 1];
+                w[k / 2] = make_float4(d.re, d.im, e.re, e.im);
+            }
+            return;
+        }
+    }
 #pragma unroll
     for (int k = 0; k < 12; ++k) {
         cplx<T> d = y.v[k] - T(0.5) * acc.v[k];
@@ -118,18 +129,19 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 384 : 128, sizeof(T) == 4 ? 2
 }
 
 template <typename T, typename Ts>
-int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const cplx<T>* b, cplx<T>* out, int nrhs,
-                  cudaStream_t st) {
+int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const cplx<T>* b, cplx<T>* out, int nrhs, cudaStream_t st,
+                  const int* lex) {
     const int ry = std::min(nrhs, sizeof(T) == 4 ? 12 : 4);  // right-hand sides per CTA
     if (g.blk44 && g.blex) {
         const dim3 grid((unsigned)g.NB * 8, (unsigned)ceil_div(nrhs, ry)), block(32, ry);
         if (b)
-            dslash44_kernel<T, Ts, true><<<grid, block, 0, st>>>(g, op, g.blex, in, b, out, nrhs);
+            dslash44_kernel<T, Ts, true><<<grid, block, 0, st>>>(g, op, g.blex, in, b, out, nrhs, lex);
         else
-            dslash44_kernel<T, Ts, false><<<grid, block, 0, st>>>(g, op, g.blex, in, b, out, nrhs);
+            dslash44_kernel<T, Ts, false><<<grid, block, 0, st>>>(g, op, g.blex, in, b, out, nrhs, lex);
         DD_CHECK_LAUNCH();
         return 0;
     }
+    if (lex) return DDAMG_ERR_INVALID_ARG;
     const dim3 grid((unsigned)ceil_div(g.V, 32), (unsigned)ceil_div(nrhs, ry)), block(32, ry);
     if (b)
         dslash_kernel<T, Ts, true><<<grid, block, 0, st>>>(g, op, in, b, out, nrhs);
@@ -140,11 +152,11 @@ int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const 
 }
 
 template int launch_dslash<double, double>(const Geom&, const FineOp<double>&, const cplx<double>*, const cplx<double>*,
-                                           cplx<double>*, int, cudaStream_t);
+                                           cplx<double>*, int, cudaStream_t, const int*);
 template int launch_dslash<double, float>(const Geom&, const FineOp<double>&, const cplx<float>*, const cplx<double>*,
-                                          cplx<double>*, int, cudaStream_t);
+                                          cplx<double>*, int, cudaStream_t, const int*);
 template int launch_dslash<float, float>(const Geom&, const FineOp<float>&, const cplx<float>*, const cplx<float>*,
-                                         cplx<float>*, int, cudaStream_t);
+                                         cplx<float>*, int, cudaStream_t, const int*);
 
 // ---------------------------------------------------------------------------
 // Red-black SAP: one launch per colour.  A CTA owns one block of that colour and

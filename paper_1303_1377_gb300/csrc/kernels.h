@@ -46,8 +46,8 @@ struct CoarseOp {
 
 // ---- fine.cu
 template <typename T, typename Ts>
-int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const cplx<T>* b, cplx<T>* out, int nrhs,
-                  cudaStream_t st);
+int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const cplx<T>* b, cplx<T>* out, int nrhs, cudaStream_t st,
+                  const int* lex = nullptr);  // lex != null (FP32, 4^4 blocks): out in the caller's layout, 16-byte aligned
 template <typename T>
 int launch_sap_colour(const Geom& g, const FineOp<T>& op, const cplx<T>* b, cplx<T>* z, int colour, int nrhs, int mr_steps,
                       cudaStream_t st);
@@ -70,6 +70,10 @@ int launch_dslash_dw(const Geom& g, const float4* U, const float2* clov, const c
 int launch_to_dw(const double* in, float2* out, size_t n, cudaStream_t st);
 int launch_clover(const Geom& g, const cplx<double>* U, double m0, double csw, double* clov, double* clovinv, cudaStream_t st);
 
+// ---- dslash44.cu: FP32 D on 4^4 blocks, two right-hand sides per thread (nrhs >= 2); lex != null: out in the
+// caller's layout (16-byte aligned)
+int launch_dslash44_pair(const Geom& g, const FineOpB& op, const cplx<float>* in, const cplx<float>* b, cplx<float>* out, const int* lex,
+                         int nrhs, cudaStream_t st);
 // ---- sap44.cu: FP32 SAP sweep on 4^4 blocks (FineOpB, FineOpB16)
 template <typename OpT>
 int launch_sap44(const Geom& g, const OpT& op, const cplx<float>* b, cplx<float>* z, int colour, int nrhs, int mr_steps, cudaStream_t st);
