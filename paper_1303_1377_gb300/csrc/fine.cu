@@ -12,7 +12,6 @@
 #include "block44.cuh"
 #include "kernels.h"
 #include "dirac.cuh"
-#include "dw.cuh"
 
 namespace ddamg {
 
@@ -806,165 +805,6 @@ int launch_clover(const Geom& g, const cplx<double>* U, double m0, double csw, d
     return 0;
 }
 
-
-// ---------------------------------------------------------------------------
-// D z for an FP32 field z with an FP64-accurate result, evaluated in double-word
-// FP32 arithmetic (pairs hi + lo of floats; error-free transformations TwoSum
-// (Knuth) and TwoProduct via FMA, as in Joldes, Muller, Popescu, "Tight and
-// rigorous error bounds for basic building blocks of double-word arithmetic",
-// ACM TOMS 2017).  Used for w = D z_k inside FGMRES, where z_k is the V-cycle
-// output and hence exactly an FP32 vector.  On GB300 an FP64 instruction costs
-// about sixty FP32 instructions, and the double-word form needs about twelve per
-// real multiply-add, with relative accuracy ~1e-14.
-// Links and site terms are stored as double-word pairs (same bytes as FP64).
-// ---------------------------------------------------------------------------
-namespace {
-
-__device__ __forceinline__ cdw ld_cdw(const float4* p) {
-    float4 v = __ldg(p);
-    return {{v.x, v.y}, {v.z, v.w}};
-}
-
-__device__ __forceinline__ cdw cdw_ipow_rt(const cdw& a, int p) {
-    cdw b = (p & 1) ? cdw{dw_neg(a.im), a.re} : a;
-    return (p & 2) ? cdw{dw_neg(b.re), dw_neg(b.im)} : b;
-}
-
-// one hop of D (direction mu, orientation fwd, given at run time) in double-word arithmetic
-__device__ __noinline__ void dw_hop_rt(cdw (&acc)[12], const cplx<float>* __restrict__ in, int V, int nb, const float4* __restrict__ U,
-                                       int link_site, int mu, bool fwd) {
-    const int c0 = c_spinb[mu][0], p0 = c_spinb[mu][1], c1 = c_spinb[mu][2], p1 = c_spinb[mu][3];
-    const int hc0 = c_spinb[mu][4], hp0 = c_spinb[mu][5], hc1 = c_spinb[mu][6], hp1 = c_spinb[mu][7];
-    cdw h[2][3];
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        cplx<float> u0 = in[(size_t)(0 * 3 + c) * V + nb], u1 = in[(size_t)(1 * 3 + c) * V + nb];
-        cplx<float> l2 = in[(size_t)(2 * 3 + c) * V + nb], l3 = in[(size_t)(3 * 3 + c) * V + nb];
-        cdw b0 = cdw_ipow_rt(c0 ? cdw{{l3.re, 0.f}, {l3.im, 0.f}} : cdw{{l2.re, 0.f}, {l2.im, 0.f}}, p0);
-        cdw b1 = cdw_ipow_rt(c1 ? cdw{{l3.re, 0.f}, {l3.im, 0.f}} : cdw{{l2.re, 0.f}, {l2.im, 0.f}}, p1);
-        cdw a0 = {{u0.re, 0.f}, {u0.im, 0.f}}, a1 = {{u1.re, 0.f}, {u1.im, 0.f}};
-        h[0][c] = fwd ? cdw_sub(a0, b0) : cdw_add(a0, b0);
-        h[1][c] = fwd ? cdw_sub(a1, b1) : cdw_add(a1, b1);
-    }
-    cdw W[9];
-#pragma unroll
-    for (int q = 0; q < 9; ++q) W[q] = ld_cdw(U + (size_t)(mu * 9 + q) * V + link_site);
-    cdw gv[2][3];
-#pragma unroll
-    for (int s = 0; s < 2; ++s) {
-#pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            cdw t = cdw_zero();
-#pragma unroll
-            for (int b = 0; b < 3; ++b) {
-                if (fwd) cdw_mac(t, W[a * 3 + b], h[s][b]);
-                else cdw_mac_conj(t, W[b * 3 + a], h[s][b]);
-            }
-            t.re = dw_norm(t.re);
-            t.im = dw_norm(t.im);
-            gv[s][a] = t;
-            acc[s * 3 + a] = cdw_add(acc[s * 3 + a], t);
-        }
-    }
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-        cdw l0 = cdw_ipow_rt(hc0 ? gv[1][c] : gv[0][c], hp0);
-        cdw l1 = cdw_ipow_rt(hc1 ? gv[1][c] : gv[0][c], hp1);
-        acc[2 * 3 + c] = fwd ? cdw_sub(acc[2 * 3 + c], l0) : cdw_add(acc[2 * 3 + c], l0);
-        acc[3 * 3 + c] = fwd ? cdw_sub(acc[3 * 3 + c], l1) : cdw_add(acc[3 * 3 + c], l1);
-    }
-}
-
-}  // namespace
-
-// thread (x, y): site blockIdx.x * 32 + x, right-hand side blockIdx.y * blockDim.y + y (the warps of
-// a CTA share the double-word links and site terms of 32 sites through L1)
-template <bool OUT_DW>
-__global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __restrict__ U, const float2* __restrict__ clov,
-                                                        const cplx<float>* __restrict__ in, void* __restrict__ outp, int nrhs) {
-    const int r = blockIdx.y * blockDim.y + threadIdx.y;
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    if (i >= g.V || r >= nrhs) return;
-    const size_t off = (size_t)r * 12 * g.V;
-    const cplx<float>* inr = in + off;
-    cdw acc[12];
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = cdw_zero();
-#pragma unroll 1
-    for (int d = 0; d < 8; ++d) {
-        const int nb = fine_nbr(g, i, d);
-        const bool fwd = (d & 1) == 0;
-        dw_hop_rt(acc, inr, g.V, nb, U, fwd ? i : nb, d >> 1, fwd);
-    }
-    // site term: y = A x with two packed hermitian 6x6 blocks (double-word entries), x FP32
-    cdw y[12];
-#pragma unroll
-    for (int h = 0; h < 2; ++h) {
-        float x[12];
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-            cplx<float> v = inr[(size_t)(h * 6 + a) * g.V + i];
-            x[2 * a] = v.re;
-            x[2 * a + 1] = v.im;
-        }
-        const float2* base = clov + (size_t)(h * 36) * g.V + i;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-            float2 dv = __ldg(base + (size_t)a * g.V);
-            dw d = {dv.x, dv.y};
-            cdw t = cdw_zero();
-            dw_macf(t.re, d, x[2 * a]);
-            dw_macf(t.im, d, x[2 * a + 1]);
-            y[h * 6 + a] = t;
-        }
-        int q = 0;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-#pragma unroll
-            for (int b = a + 1; b < 6; ++b) {
-                float2 mr = __ldg(base + (size_t)(6 + 2 * q) * g.V), mi = __ldg(base + (size_t)(7 + 2 * q) * g.V);
-                dw m_re = {mr.x, mr.y}, m_im = {mi.x, mi.y};
-                // y[a] += m x[b];  y[b] += conj(m) x[a]
-                dw_macf(y[h * 6 + a].re, m_re, x[2 * b]);
-                dw_macf(y[h * 6 + a].re, dw_neg(m_im), x[2 * b + 1]);
-                dw_macf(y[h * 6 + a].im, m_re, x[2 * b + 1]);
-                dw_macf(y[h * 6 + a].im, m_im, x[2 * b]);
-                dw_macf(y[h * 6 + b].re, m_re, x[2 * a]);
-                dw_macf(y[h * 6 + b].re, m_im, x[2 * a + 1]);
-                dw_macf(y[h * 6 + b].im, m_re, x[2 * a + 1]);
-                dw_macf(y[h * 6 + b].im, dw_neg(m_im), x[2 * a]);
-                ++q;
-            }
-        }
-    }
-    if (OUT_DW) {
-        float4* o = reinterpret_cast<float4*>(outp) + off;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            dw re = dw_norm(dw_add(y[k].re, {-0.5f * acc[k].re.h, -0.5f * acc[k].re.l}));
-            dw im = dw_norm(dw_add(y[k].im, {-0.5f * acc[k].im.h, -0.5f * acc[k].im.l}));
-            o[(size_t)k * g.V + i] = make_float4(re.h, re.l, im.h, im.l);
-        }
-    } else {
-        cplx<double>* o = reinterpret_cast<cplx<double>*>(outp) + off;
-#pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            double re = (double)y[k].re.h + (double)y[k].re.l - 0.5 * ((double)acc[k].re.h + (double)acc[k].re.l);
-            double im = (double)y[k].im.h + (double)y[k].im.l - 0.5 * ((double)acc[k].im.h + (double)acc[k].im.l);
-            o[(size_t)k * g.V + i] = mk(re, im);
-        }
-    }
-}
-
-int launch_dslash_dw(const Geom& g, const float4* U, const float2* clov, const cplx<float>* in, void* out, bool out_dw, int nrhs,
-                     cudaStream_t st) {
-    const int ry = std::min(nrhs, 4);
-    const dim3 grid((unsigned)ceil_div(g.V, 32), (unsigned)ceil_div(nrhs, ry)), block(32, ry);
-    if (out_dw) dslash_dw_kernel<true><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
-    else dslash_dw_kernel<false><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
-    DD_CHECK_LAUNCH();
-    return 0;
-}
 
 // FP64 array -> double-word pairs (hi = nearest float, lo = nearest float of the remainder)
 __global__ void to_dw_kernel(const double* __restrict__ in, float2* __restrict__ out, size_t n) {

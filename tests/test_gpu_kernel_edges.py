@@ -104,3 +104,20 @@ def test_fp32_dslash_by_right_hand_sides_and_alignment(dims, nrhs):
     for r in range(nrhs):
         ref = D.apply(x[r].astype(np.complex128))
         assert np.max(np.abs(got[r].cpu().numpy() - ref)) < 1e-6 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dims,block,nrhs", [((8, 8, 8, 8), (4, 4, 4, 4), 1), ((8, 4, 4, 12), (4, 2, 2, 2), 2), ((8, 8, 8, 16), (4, 4, 4, 4), 9)])
+def test_double_word_dslash_by_right_hand_sides(dims, block, nrhs):
+    """D in double-word arithmetic, one field and pairs (odd and even batches): the stated 1e-13 against the
+    oracle's FP64."""
+    from oracle.dirac import DiracOperator
+    from paper_1303_1377_gb300 import ddamg
+
+    s, U = _solver(dims, n_vec=4, block=block, precision=ddamg.PREC_SINGLE)
+    with s:
+        x = synth.gaussian_spinors(dims, nrhs, seed=51).astype(np.complex64)
+        got = s.apply_D_mixed(x)
+    D = DiracOperator(U, dims, -0.4, 1.0)
+    for r in range(nrhs):
+        ref = D.apply(x[r].astype(np.complex128))
+        assert np.max(np.abs(got[r] - ref)) < 1e-13 * np.max(np.abs(ref))
