@@ -243,68 +243,18 @@ int gauge_to_internal(const cplx<double>* in, cplx<double>* out, const int* lex_
 
 // Hessenberg bookkeeping of batched (F)GMRES: one thread per right-hand side (the update: one warp).
 // Column k of H arrives in hcol[i * nrhs + r] (i <= k) with ||w||^2 in hcol[(k+1) * nrhs + r].re.
-// One warp per right-hand side: the lanes fetch the new Hessenberg column and the stored rotations
-// side by side into shared memory, lane 0 applies the rotations in order (the only sequential part),
-// and the lanes write the column back.
-constexpr int kArnoldiMaxM = 64;
 __global__ void __launch_bounds__(32) arnoldi_update_kernel(KrylovState s, int k, const cplx<double>* __restrict__ hcol,
                                                             cplx<double>* __restrict__ scale) {
     const int r = blockIdx.x, lane = threadIdx.x;
-    const int m = s.m;
-    cplx<double>* H = s.H + (size_t)r * (m + 1) * m;  // H[i * m + k]
     if (!s.active[r]) {
         if (lane == 0) scale[r] = mk(0.0, 0.0);
         return;
     }
-    __shared__ cplx<double> col[kArnoldiMaxM + 1], sn_s[kArnoldiMaxM];
-    __shared__ double cs_s[kArnoldiMaxM];
-    for (int i = lane; i <= k + 1; i += 32) col[i] = hcol[(size_t)i * s.nrhs + r];
-    for (int i = lane; i < k; i += 32) {
-        cs_s[i] = s.cs[r * m + i];
-        sn_s[i] = s.sn[r * m + i];
-    }
+    __shared__ ArnoldiWork w;
+    for (int i = lane; i <= k + 1; i += 32) w.col[i] = hcol[(size_t)i * s.nrhs + r];
     __syncwarp();
-    if (lane == 0) {
-        const double hk = sqrt(col[k + 1].re);
-        // apply the previous rotations
-        for (int i = 0; i < k; ++i) {
-            const double c = cs_s[i];
-            const cplx<double> sn = sn_s[i];
-            const cplx<double> a = col[i], b = col[i + 1];
-            col[i] = c * a + sn * b;
-            col[i + 1] = c * b - conj(sn) * a;
-        }
-        const cplx<double> a = col[k];
-        const double na = sqrt(norm2(a));
-        const double den = sqrt(na * na + hk * hk);
-        double c;
-        cplx<double> sn;
-        if (den == 0.0) {
-            c = 1.0;
-            sn = mk(0.0, 0.0);
-        } else if (na == 0.0) {
-            c = 0.0;
-            sn = mk(1.0, 0.0);
-        } else {
-            c = na / den;
-            sn = (hk / (na * den)) * a;  // (a/|a|) conj(hk)/den, hk real
-        }
-        s.cs[r * m + k] = c;
-        s.sn[r * m + k] = sn;
-        col[k] = c * a + hk * sn;
-        const cplx<double> gk = s.g[r * (m + 1) + k];
-        s.g[r * (m + 1) + k + 1] = -1.0 * (conj(sn) * gk);
-        s.g[r * (m + 1) + k] = c * gk;
-        const double est = sqrt(norm2(s.g[r * (m + 1) + k + 1]));
-        s.steps[r] = k + 1;
-        s.resid[r] = est;
-        const bool nonfinite = !(est == est) || !(hk == hk);
-        if (nonfinite) s.flags[r] |= 2;
-        if (est <= s.ctarget[r] || nonfinite) s.active[r] = 0;
-        scale[r] = (hk > 0.0 && s.active[r]) ? mk(1.0 / hk, 0.0) : mk(0.0, 0.0);
-    }
-    __syncwarp();
-    for (int i = lane; i <= k; i += 32) H[i * m + k] = col[i];
+    const double sc = arnoldi_column(s, r, k, lane, w);
+    if (lane == 0) scale[r] = mk(sc, 0.0);
 }
 
 // y = H^{-1} g (upper triangular, steps[r] columns); y stored as coef[i * nrhs + r]

@@ -23,6 +23,77 @@ struct KrylovState {
     double cycle_tol;  // 0: a cycle runs to target (or the restart length)
 };
 
+// One Arnoldi step's Hessenberg column of right-hand side r, by one warp: w.col[0..k] = <V_i, w>, w.col[k+1].re =
+// ||w||^2.  Rotates the column by the stored Givens rotations, forms the new one, updates the residual estimate
+// and the flags, and returns on every lane the factor that normalises w (0: the right-hand side has converged or
+// broken down).  An FP64 instruction occupies the warp's unit for 64 cycles whatever the number of active lanes
+// (1/64 of the FP32 rate), so what the rotations do not chain is spread over the lanes: of a rotation only the
+// running entry r <- c_i col_{i+1} - conj(sn_i) r is sequential (lane parity = real / imaginary part: two
+// multiply-adds and a shuffle), and the square roots and quotients run side by side in four lanes.  One lane
+// doing all of it took about 1 us per rotation and 10 us besides.
+constexpr int kArnoldiMaxM = 64;
+struct ArnoldiWork {
+    cplx<double> col[kArnoldiMaxM + 1], sn[kArnoldiMaxM], d[kArnoldiMaxM], run[kArnoldiMaxM + 1];
+    double cs[kArnoldiMaxM];
+};
+__device__ __forceinline__ double arnoldi_column(const KrylovState& s, int r, int k, int lane, ArnoldiWork& w) {
+    const int m = s.m;
+    cplx<double>* H = s.H + (size_t)r * (m + 1) * m;  // H[i * m + k]
+    const cplx<double> gk = s.g[r * (m + 1) + k];
+    const double prev = s.resid[r], ctarget = s.ctarget[r];  // prev = |g_k|
+    for (int i = lane; i < k; i += 32) {
+        w.cs[i] = s.cs[r * m + i];
+        w.sn[i] = s.sn[r * m + i];
+    }
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) w.d[i] = w.cs[i] * w.col[i + 1];
+    const int part = lane & 1;
+    double x = part ? w.col[0].im : w.col[0].re;
+    __syncwarp();
+    for (int i = 0; i < k; ++i) {
+        const double y = __shfl_xor_sync(0xffffffffu, x, 1);
+        const cplx<double> sn = w.sn[i];
+        if (lane < 2) reinterpret_cast<double*>(&w.run[i])[part] = x;
+        x = fma(part ? sn.im : -sn.im, y, fma(-sn.re, x, part ? w.d[i].im : w.d[i].re));
+    }
+    const double y = __shfl_xor_sync(0xffffffffu, x, 1);
+    const cplx<double> a = part ? mk(y, x) : mk(x, y);
+    __syncwarp();
+    for (int i = lane; i < k; i += 32) H[i * m + k] = w.cs[i] * w.run[i] + w.sn[i] * w.col[i + 1];
+    const double n2 = w.col[k + 1].re, a2 = norm2(a);
+    const double root = sqrt(lane == 0 ? n2 : lane == 1 ? a2 : a2 + n2);
+    const double hk = __shfl_sync(0xffffffffu, root, 0), na = __shfl_sync(0xffffffffu, root, 1), den = __shfl_sync(0xffffffffu, root, 2);
+    const double quot = (lane == 0 ? 1.0 : lane == 1 ? na : hk) / (lane == 0 ? hk : lane == 2 ? na * den : den);
+    const double inv = __shfl_sync(0xffffffffu, quot, 0), q1 = __shfl_sync(0xffffffffu, quot, 1), q2 = __shfl_sync(0xffffffffu, quot, 2),
+                 q3 = __shfl_sync(0xffffffffu, quot, 3);
+    double sc = 0.0;
+    if (lane == 0) {
+        double c = q1, red = q3;
+        cplx<double> sn = q2 * a;  // (a/|a|) conj(hk)/den, hk real
+        if (den == 0.0) c = 1.0, red = 0.0, sn = mk(0.0, 0.0);
+        else if (na == 0.0) c = 0.0, red = 1.0, sn = mk(1.0, 0.0);
+        s.cs[r * m + k] = c;
+        s.sn[r * m + k] = sn;
+        H[k * m + k] = c * a + hk * sn;
+        s.g[r * (m + 1) + k + 1] = -1.0 * (conj(sn) * gk);
+        s.g[r * (m + 1) + k] = c * gk;
+        const double est = red * prev;  // |g_{k+1}| = |sn| |g_k|
+        s.steps[r] = k + 1;
+        s.resid[r] = est;
+        const bool nonfinite = !(est == est) || !(hk == hk);
+        if (nonfinite) s.flags[r] |= 2;
+        const bool done = est <= ctarget || nonfinite;
+        if (done) s.active[r] = 0;
+        sc = hk > 0.0 && !done ? inv : 0.0;
+    }
+    return __shfl_sync(0xffffffffu, sc, 0);
+}
+
+// One Arnoldi step on short FP32 vectors (ortho.cu): V_{k+1} holds A V_k on entry and the next basis vector
+// on exit; the Hessenberg column, the residual estimate and the flags of s are updated.
+bool ortho_step_supported(const cplx<float>* V, size_t bstride, size_t n, int k);
+int ortho_step_f32(const KrylovState& s, int k, cplx<float>* V, size_t bstride, size_t n, cudaStream_t st);
+
 template <typename Ta, typename Tb>
 int multidot(const cplx<Ta>* A, size_t istride, size_t arstride, int k, const cplx<Tb>* w, size_t wrstride, size_t n, int nrhs,
              cplx<double>* out, int ostride_i, double* scratch, cudaStream_t st);

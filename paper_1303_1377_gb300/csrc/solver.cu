@@ -919,6 +919,10 @@ static int krylov(ddamg_handle* h, KrylovBufs& kb, KrylovProblem<TB, TV, TZ>& P,
                     DD_TRY(P.A(zk, wk));
                     const double vb = (double)sizeof(cplx<TV>) * n * nr;
                     Prof pr(h, PF_ORTHO, vb * (2 * (k + 1) + 6));
+                    if constexpr (std::is_same<TV, float>::value) {
+                        if (!P.reorth && ortho_step_supported(P.Vb, bstride, n, k))  // short vectors: one kernel
+                            return ortho_step_f32(s, k, P.Vb, bstride, n, st);
+                    }
                     // the last product is ||w||^2 before orthogonalisation, kept for the DGKS test
                     DD_TRY(lean_multidot(P.Vb, bstride, n, k + 2, wk, nr, kb.hcol, kb, nullptr, st, kb.nbefore));
                     DD_TRY(lean_axpy_norm(wk, P.Vb, bstride, n, k + 1, kb.hcol, nr, kb, kb.hcol + (size_t)(k + 1) * nr, nullptr, st));

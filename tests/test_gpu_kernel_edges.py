@@ -121,3 +121,23 @@ def test_double_word_dslash_by_right_hand_sides(dims, block, nrhs):
     for r in range(nrhs):
         ref = D.apply(x[r].astype(np.complex128))
         assert np.max(np.abs(got[r] - ref)) < 1e-13 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dims,block,n_vec,nrhs,steps", [((4, 4, 4, 4), (2, 2, 2, 2), 1, 3, 5), ((4, 4, 4, 8), (2, 2, 2, 2), 3, 1, 9),
+                                                         ((8, 8, 8, 16), (2, 2, 2, 4), 5, 13, 35), ((16, 16, 16, 8), (2, 2, 2, 2), 10, 2, 12)])
+def test_coarse_gmres_steps_by_vector_length(dims, block, n_vec, nrhs, steps):
+    """A fixed number of FP32 coarse GMRES steps on vectors of 16 to 20480 numbers (slices with idle CTAs, a
+    ragged last slice, a restart, and beyond the one-kernel step) against FP64 steps on the same operator, to
+    the stated 1e-6.  Random test vectors keep the coarse operator well conditioned."""
+    from paper_1303_1377_gb300 import ddamg
+
+    v = synth.random_test_vectors(dims, n_vec, seed=61)
+    out = {}
+    for prec in ("DOUBLE", "SINGLE"):
+        s, _ = _solver(dims, n_vec=n_vec, block=block, precision=getattr(ddamg, "PREC_" + prec))
+        with s:
+            s.setup_from_vectors(v)
+            e = synth.gaussian_coarse(s.n_coarse, s.coarse_dof, nrhs, seed=62)
+            out[prec] = s.coarse_solve(e, steps)
+    for r in range(nrhs):
+        assert np.max(np.abs(out["SINGLE"][r] - out["DOUBLE"][r])) < 1e-6 * np.max(np.abs(out["DOUBLE"][r]))
