@@ -53,20 +53,23 @@ __global__ void __launch_bounds__(kDotThreads) multidot_kernel(const cplx<Ta>* _
     }
 }
 
-// stage 2: out[i * ostride_i + r] = sum over the ctas of rhs r
-__global__ void multidot_finish(const double* __restrict__ partial, int k, int nrhs, int ctas_per_rhs,
-                                cplx<double>* __restrict__ out, int ostride_i, const int* __restrict__ run_flag = nullptr) {
+// stage 2: out[i * ostride_i + r] = sum over the ctas of rhs r.  One warp per product, the CTAs' partial sums side
+// by side in a fixed order (one thread per product took 16 us for 1216 CTAs, a chain of loads and FP64 additions).
+__global__ void __launch_bounds__(128) multidot_finish(const double* __restrict__ partial, int k, int nrhs, int ctas_per_rhs,
+                                                       cplx<double>* __restrict__ out, int ostride_i,
+                                                       const int* __restrict__ run_flag = nullptr) {
     if (run_flag && !*run_flag) return;
-    int q = blockIdx.x * blockDim.x + threadIdx.x;  // q = r * k + i
+    const int q = blockIdx.x * 4 + (threadIdx.x >> 5), lane = threadIdx.x & 31;  // q = r * k + i
     if (q >= nrhs * k) return;
-    int r = q / k, i = q % k;
+    const int r = q / k, i = q % k;
     double re = 0, im = 0;
-    for (int p = 0; p < ctas_per_rhs; ++p) {
+    for (int p = lane; p < ctas_per_rhs; p += 32) {
         const double* src = partial + ((size_t)(p * nrhs + r)) * 2 * k;
         re += src[2 * i];
         im += src[2 * i + 1];
     }
-    out[(size_t)i * ostride_i + r] = mk(re, im);
+    re = warp_sum(re), im = warp_sum(im);
+    if (lane == 0) out[(size_t)i * ostride_i + r] = mk(re, im);
 }
 
 template <typename Ta, typename Tb>
@@ -92,7 +95,7 @@ int multidot(const cplx<Ta>* A, size_t istride, size_t arstride, int k, const cp
         else
             multidot_kernel<Ta, Tb, 32><<<ctas * nrhs, kDotThreads, 0, st>>>(Ab, istride, arstride, kk, w, wrstride, n, nrhs, ctas, scratch);
         DD_CHECK_LAUNCH();
-        multidot_finish<<<ceil_div((long long)nrhs * kk, 128), 128, 0, st>>>(scratch, kk, nrhs, ctas, out + (size_t)off * ostride_i,
+        multidot_finish<<<ceil_div((long long)nrhs * kk, 4), 128, 0, st>>>(scratch, kk, nrhs, ctas, out + (size_t)off * ostride_i,
                                                                           ostride_i);
         DD_CHECK_LAUNCH();
         off += kk;
@@ -257,20 +260,31 @@ __global__ void __launch_bounds__(32) arnoldi_update_kernel(KrylovState s, int k
     if (lane == 0) scale[r] = mk(sc, 0.0);
 }
 
-// y = H^{-1} g (upper triangular, steps[r] columns); y stored as coef[i * nrhs + r]
-__global__ void arnoldi_solve_kernel(KrylovState s, cplx<double>* __restrict__ y) {
-    int r = blockIdx.x * blockDim.x + threadIdx.x;
-    if (r >= s.nrhs) return;
-    const int m = s.m;
+// y = H^{-1} g (upper triangular, steps[r] columns); y stored as coef[i * nrhs + r].  One warp per right-hand
+// side: the triangle and the reciprocals of its diagonal are fetched and formed side by side, and a step of the
+// back-substitution updates all remaining rows at once (one thread walking the triangle through global memory
+// took 17 us for eight columns).
+__global__ void __launch_bounds__(32) arnoldi_solve_kernel(KrylovState s, cplx<double>* __restrict__ y) {
+    const int r = blockIdx.x, lane = threadIdx.x, m = s.m;
     const cplx<double>* H = s.H + (size_t)r * (m + 1) * m;
-    int n = s.steps[r];
-    for (int i = m - 1; i >= n; --i) y[(size_t)i * s.nrhs + r] = mk(0.0, 0.0);
+    __shared__ cplx<double> R[kArnoldiMaxM * (kArnoldiMaxM + 1) / 2];  // column i: R[i (i + 1) / 2 + j], j <= i
+    __shared__ cplx<double> t[kArnoldiMaxM], inv[kArnoldiMaxM];
+    const int n = s.steps[r];
+    for (int i = n + lane; i < m; i += 32) y[(size_t)i * s.nrhs + r] = mk(0.0, 0.0);
+    for (int i = 0; i < n; ++i)
+        for (int j = lane; j <= i; j += 32) R[i * (i + 1) / 2 + j] = H[j * m + i];
+    for (int i = lane; i < n; i += 32) {
+        t[i] = s.g[r * (m + 1) + i];
+        const cplx<double> d = H[i * m + i];
+        const double dn = norm2(d);
+        inv[i] = dn > 0 ? mk(d.re / dn, -d.im / dn) : mk(0.0, 0.0);
+    }
+    __syncwarp();
     for (int i = n - 1; i >= 0; --i) {
-        cplx<double> t = s.g[r * (m + 1) + i];
-        for (int j = i + 1; j < n; ++j) t = t - H[i * m + j] * y[(size_t)j * s.nrhs + r];
-        cplx<double> d = H[i * m + i];
-        double dn = norm2(d);
-        y[(size_t)i * s.nrhs + r] = dn > 0 ? t * mk(d.re / dn, -d.im / dn) : mk(0.0, 0.0);
+        const cplx<double> yi = t[i] * inv[i];
+        if (lane == 0) y[(size_t)i * s.nrhs + r] = yi;
+        for (int j = lane; j < i; j += 32) t[j] = t[j] - R[i * (i + 1) / 2 + j] * yi;
+        __syncwarp();
     }
 }
 
@@ -304,7 +318,8 @@ int arnoldi_update(const KrylovState& s, int k, const cplx<double>* hcol, cplx<d
     return 0;
 }
 int arnoldi_solve(const KrylovState& s, cplx<double>* y, cudaStream_t st) {
-    arnoldi_solve_kernel<<<ceil_div(s.nrhs, 64), 64, 0, st>>>(s, y);
+    if (s.m > kArnoldiMaxM) return DDAMG_ERR_INVALID_ARG;
+    arnoldi_solve_kernel<<<s.nrhs, 32, 0, st>>>(s, y);
     DD_CHECK_LAUNCH();
     return 0;
 }
@@ -382,7 +397,7 @@ int multidot_dw(const cplx<dwf>* A, size_t istride, size_t arstride, int k, cons
         else
             multidot_dw_kernel<16><<<ctas * nrhs, kDotThreads, 0, st>>>(Ab, istride, arstride, kk, w, wrstride, n, nrhs, ctas, scratch, run_flag);
         DD_CHECK_LAUNCH();
-        multidot_finish<<<ceil_div((long long)nrhs * kk, 128), 128, 0, st>>>(scratch, kk, nrhs, ctas, out + (size_t)off * ostride_i,
+        multidot_finish<<<ceil_div((long long)nrhs * kk, 4), 128, 0, st>>>(scratch, kk, nrhs, ctas, out + (size_t)off * ostride_i,
                                                                           ostride_i, run_flag);
         DD_CHECK_LAUNCH();
         off += kk;
@@ -487,7 +502,7 @@ int axpy_norm_dw(cplx<dwf>* w, const cplx<dwf>* A, size_t istride, size_t rstrid
     if (ctas > target) ctas = target;
     axpy_norm_dw_kernel<<<ctas * nrhs, kAxpyThreads, 0, st>>>(w, A, istride, rstride, k, coef_scratch, n, nrhs, ctas, scratch, run_flag);
     DD_CHECK_LAUNCH();
-    multidot_finish<<<ceil_div((long long)nrhs, 128), 128, 0, st>>>(scratch, 1, nrhs, ctas, norm_out, nrhs, run_flag);
+    multidot_finish<<<ceil_div((long long)nrhs, 4), 128, 0, st>>>(scratch, 1, nrhs, ctas, norm_out, nrhs, run_flag);
     DD_CHECK_LAUNCH();
     return 0;
 }
