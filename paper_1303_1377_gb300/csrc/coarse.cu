@@ -7,6 +7,8 @@
 // Coarse sites in internal order: even (red) sites first, then odd.
 // Vectors: cplx[nrhs][sites][nc] addressed through (pointer, rhs stride,
 // first site) so that half vectors and full vectors share one kernel.
+#include <algorithm>
+
 #include "kernels.h"
 
 namespace ddamg {
@@ -39,7 +41,7 @@ __device__ __forceinline__ void gemm_slice(const S* first, int nc, int p, int q0
                                            cplx<T> (&acc)[2][NRP]) {
     const S* bp = first + 2 * ((size_t)q0 * nc + 2 * p);
     const cplx<T>* xq = xs + (size_t)q0 * NRP;
-#pragma unroll 2
+#pragma unroll(NRP == 1 ? 4 : 2)
     for (int q = q0; q < q1; ++q, bp += 2 * nc, xq += NRP) {
         cplx<T> b0, b1;
         load_pair(bp, b0, b1);
@@ -56,8 +58,11 @@ __device__ __forceinline__ void gemm_slice(const S* first, int nc, int p, int q0
 // k-group g of the 8 or 9 (direction, column) slices; partial sums are reduced in
 // shared memory.  acc = self + hop_sign * sum_{d=1..8} B_d(c) xin[nbr_d(c)] with
 //   self = 0 (self_mode 0), B_0(c) xself[c] (1) or xself[c] (2);  out = apply_inv ? Dinv acc : acc.
-template <typename T, typename S, int NRP>
-__global__ void __launch_bounds__(128) coarse_stencil_kernel(CoarseOp<S> op, int site_begin, CVec<T> xin, CVec<T> xself,
+// WIDE (few sites, one or two right-hand sides): 1024 threads per CTA.  Such a launch is bound by the latency of
+// the matrix columns a thread reads one after the other (60 of them at 2N = 40 with 128 threads, 8 with 1024),
+// and there are not enough sites for more CTAs.
+template <typename T, typename S, int NRP, bool WIDE>
+__global__ void __launch_bounds__(WIDE ? 1024 : 128) coarse_stencil_kernel(CoarseOp<S> op, int site_begin, CVec<T> xin, CVec<T> xself,
                                                              int self_mode, T hop_sign, int apply_inv, CVec<T> out, int nrhs) {
     extern __shared__ unsigned char smem_raw[];
     const int nc = op.nc, RP = nc / 2;
@@ -91,6 +96,34 @@ __global__ void __launch_bounds__(128) coarse_stencil_kernel(CoarseOp<S> op, int
 #pragma unroll
         for (int r = 0; r < NRP; ++r) acc[h][r] = czero<T>();
     const int Kt = nslots * nc;
+    // vsum[o] = sum of the KG partial sums red[g][o] (+ what self adds)
+    auto reduce = [&](const cplx<T>* red, cplx<T>* vsum, bool self) {
+        const int tot = nc * NRP;
+        auto put = [&](int o, cplx<T> s) {
+            if (self) {
+                const int row = o / NRP, r = o % NRP;
+                if (r < nrhs) s = s + xself.p[r * xself.rstride + (size_t)(c - xself.site0) * nc + row];
+            }
+            vsum[o] = s;
+        };
+        if constexpr (WIDE) {  // eight lanes per output
+            for (int o0 = 0; o0 < tot; o0 += blockDim.x / 8) {
+                const int o = o0 + threadIdx.x / 8, l8 = threadIdx.x & 7;
+                cplx<T> s = czero<T>();
+                if (o < tot)
+                    for (int gg = l8; gg < KG; gg += 8) s = s + red[(size_t)gg * tot + o];
+#pragma unroll
+                for (int m = 1; m < 8; m <<= 1) s = s + mk(__shfl_xor_sync(0xffffffffu, s.re, m), __shfl_xor_sync(0xffffffffu, s.im, m));
+                if (l8 == 0 && o < tot) put(o, s);
+            }
+        } else {
+            for (int o = threadIdx.x; o < tot; o += blockDim.x) {
+                cplx<T> s = czero<T>();
+                for (int gg = 0; gg < KG; ++gg) s = s + red[(size_t)gg * tot + o];
+                put(o, s);
+            }
+        }
+    };
     if (act && nslots > 0) gemm_slice<T, S, NRP>(first, nc, p, (g * Kt) / KG, ((g + 1) * Kt) / KG, xs, acc);
     __syncthreads();
     // reduce the KG partial sums: red[g][row][r]
@@ -103,15 +136,7 @@ __global__ void __launch_bounds__(128) coarse_stencil_kernel(CoarseOp<S> op, int
         }
     __syncthreads();
     cplx<T>* vsum = red + (size_t)KG * nc * NRP;  // [nc][NRP]
-    for (int o = threadIdx.x; o < nc * NRP; o += blockDim.x) {
-        cplx<T> s = czero<T>();
-        for (int gg = 0; gg < KG; ++gg) s = s + red[(size_t)gg * nc * NRP + o];
-        if (self_mode == 2) {
-            int row = o / NRP, r = o % NRP;
-            if (r < nrhs) s = s + xself.p[r * xself.rstride + (size_t)(c - xself.site0) * nc + row];
-        }
-        vsum[o] = s;
-    }
+    reduce(red, vsum, self_mode == 2);
     __syncthreads();
     if (apply_inv) {
         const S* dfirst = op.Dinv + ((size_t)c * nc) * nc * 2;
@@ -128,11 +153,7 @@ __global__ void __launch_bounds__(128) coarse_stencil_kernel(CoarseOp<S> op, int
                 red[((size_t)g * nc + 2 * p + 1) * NRP + r] = acc[1][r];
             }
         __syncthreads();
-        for (int o = threadIdx.x; o < nc * NRP; o += blockDim.x) {
-            cplx<T> s = czero<T>();
-            for (int gg = 0; gg < KG; ++gg) s = s + red[(size_t)gg * nc * NRP + o];
-            vsum[o] = s;
-        }
+        reduce(red, vsum, false);
         __syncthreads();
     }
     for (int o = threadIdx.x; o < nc * NRP; o += blockDim.x) {
@@ -141,25 +162,37 @@ __global__ void __launch_bounds__(128) coarse_stencil_kernel(CoarseOp<S> op, int
     }
 }
 
-template <typename T, typename S, int NRP>
-static int launch_stencil_nrp(const CoarseOp<S>& op, int site_begin, int nsites, CVec<T> xin, CVec<T> xself, int self_mode,
-                              T hop_sign, int apply_inv, CVec<T> out, int nrhs, cudaStream_t st) {
+template <typename T, typename S, int NRP, bool WIDE>
+static int launch_stencil_threads(const CoarseOp<S>& op, int site_begin, int nsites, CVec<T> xin, CVec<T> xself, int self_mode,
+                                  T hop_sign, int apply_inv, CVec<T> out, int nrhs, cudaStream_t st) {
     const int RP = op.nc / 2;
-    int KG = 128 / RP;
-    if (KG < 1) KG = 1;
-    const int nt = KG * RP;
+    // whole warps; the threads past KG * RP only help with staging and sums
+    const int nt = WIDE ? 1024 : (std::max(RP, 128 / RP * RP) + 31) & ~31;
+    const int KG = nt / RP;
     size_t stage = (size_t)9 * op.nc * NRP * sizeof(cplx<T>);
     size_t reduce = (size_t)(KG + 1) * op.nc * NRP * sizeof(cplx<T>);
     size_t smem = stage > reduce ? stage : reduce;
     // set once per kernel instance (a function-local static initialiser is thread safe)
     static const bool attr = [] {
-        cudaFuncSetAttribute(coarse_stencil_kernel<T, S, NRP>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(coarse_stencil_kernel<T, S, NRP, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         return true;
     }();
     (void)attr;
-    coarse_stencil_kernel<T, S, NRP><<<nsites, nt, smem, st>>>(op, site_begin, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs);
+    coarse_stencil_kernel<T, S, NRP, WIDE><<<nsites, nt, smem, st>>>(op, site_begin, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs);
     DD_CHECK_LAUNCH();
     return 0;
+}
+template <typename T, typename S, int NRP>
+static int launch_stencil_nrp(const CoarseOp<S>& op, int site_begin, int nsites, CVec<T> xin, CVec<T> xself, int self_mode,
+                              T hop_sign, int apply_inv, CVec<T> out, int nrhs, cudaStream_t st) {
+    // FP32, 2N = 40, us per launch wide / narrow: one right-hand side 9.3 / 17.0 (8 sites), 9.9 / 17.9 (128), 11.5 /
+    // 18.0 (256); two 11.3 / 14.0 (8), 11.4 / 14.3 (128), 17.0 / 14.9 (256); four 14.8 / 16.2 (8), 25.6 / 18.6 (256).
+    // FP64: one 27.7 / 30.9 (128), two 44.9 / 44.6.
+    if constexpr (NRP == 1 || (NRP == 2 && sizeof(T) == 4)) {
+        if (nsites <= 152 * (NRP == 1 ? 2 : 1))
+            return launch_stencil_threads<T, S, NRP, true>(op, site_begin, nsites, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs, st);
+    }
+    return launch_stencil_threads<T, S, NRP, false>(op, site_begin, nsites, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs, st);
 }
 
 // batch of up to kMaxCoarseBatch right-hand sides per launch; larger batches are split
