@@ -1189,14 +1189,16 @@ static int build_interpolation(ddamg_handle* h) {
     DD_TRY(tscr.ensure(sizeof(cplx<double>) * fld * chunk));
     FineOp<double> op64{h->U64, h->clov64, h->clovinv64};
     int rc = 0;
-    for (int dir = 0; dir < 9 && !rc; ++dir)
+    for (int dir = 0; dir < 9 && !rc; dir += dir == 0 ? 1 : 2)  // self and the four forward directions
         for (int col0 = 0; col0 < 2 * N && !rc; col0 += chunk) {
             const int ncols = std::min(chunk, 2 * N - col0);
-            rc = launch_assemble_T(h->g, op64, h->P64, N, dir, col0, ncols, tscr.as<cplx<double>>(), st);
+            rc = launch_assemble_T(h->g, op64, h->P64, N, dir, col0, ncols, h->d_sites + (size_t)dir * h->Vb, h->nsites[dir],
+                                   tscr.as<cplx<double>>(), st);
             if (!rc)
                 rc = launch_block_project(h->g, h->P64, N, tscr.as<cplx<double>>(), col0, ncols, h->d_sites + (size_t)dir * h->Vb,
                                           h->nsites[dir], h->B64 + (size_t)dir * nc * nc * 2, (size_t)9 * nc * nc, st);
         }
+    if (!rc) rc = launch_complete_stencil(h->g, N, h->B64, st);
     DD_CUDA(cudaStreamSynchronize(st));
     tscr.release();
     if (rc) return rc;

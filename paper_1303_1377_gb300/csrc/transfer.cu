@@ -212,6 +212,7 @@ template int launch_prolong<float, float>(const Geom&, const cplx<float>*, int, 
 // local orthonormalisation (Sec. 3.1): modified Gram-Schmidt of P_1..P_N on every
 // aggregate (block c, half h), in place, FP64.  CTA = (c, h), thread = site.
 // ---------------------------------------------------------------------------
+constexpr int kMaxVec = 32;  // params.n_vec is at most 32
 __device__ __forceinline__ double block_sum_d(double v, double* red) {
     v = warp_sum(v);
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
@@ -223,133 +224,257 @@ __device__ __forceinline__ double block_sum_d(double v, double* red) {
     return s;
 }
 
-__global__ void gram_schmidt_kernel(Geom g, cplx<double>* __restrict__ P, int N, int* __restrict__ fail) {
-    __shared__ double red[32];
+// Right-looking: once p_j is normalised, all later vectors are projected against it, eight at a time, so that
+// one block reduction serves eight inner products; each vector meets p_0, p_1, ... in the same order as in the
+// left-looking form.  Bound by FP64 arithmetic (N^2 / 2 products and updates of 6 Vb components per aggregate
+// half): 20 vectors on 16^4 5.08 -> 2.93 ms, where the left-looking form waited for two block reductions per
+// pair of vectors.
+template <int MAXT>
+__global__ void __launch_bounds__(MAXT) gram_schmidt_kernel(Geom g, cplx<double>* __restrict__ P, int N, int* __restrict__ fail) {
+    constexpr int Q = 8, K = 2 * Q;  // vectors and real numbers per reduction
+    __shared__ double red[32], part[32][K], tot[K], orig_s[kMaxVec];
     const int c = blockIdx.x >> 1, h = blockIdx.x & 1;
-    const int l = threadIdx.x;
+    const int l = threadIdx.x, w = l >> 5, lane = l & 31, nw = blockDim.x >> 5;
     const bool act = l < g.Vb;
-    const int i = c * g.Vb + l;
-    for (int j = 0; j < N; ++j) {
-        cplx<double>* pj = P + (size_t)j * 12 * g.V;
-        double orig = 0;
-        if (act)
-            for (int k = 6 * h; k < 6 * h + 6; ++k) orig += norm2(pj[(size_t)k * g.V + i]);
-        orig = block_sum_d(orig, red);
-        for (int q = 0; q < j; ++q) {
-            const cplx<double>* pq = P + (size_t)q * 12 * g.V;
-            cplx<double> d = czero<double>();
-            if (act)
-                for (int k = 6 * h; k < 6 * h + 6; ++k) cmac_conj(d, pq[(size_t)k * g.V + i], pj[(size_t)k * g.V + i]);
-            d.re = block_sum_d(d.re, red);
-            d.im = block_sum_d(d.im, red);
-            if (act)
-                for (int k = 6 * h; k < 6 * h + 6; ++k) pj[(size_t)k * g.V + i] = pj[(size_t)k * g.V + i] - d * pq[(size_t)k * g.V + i];
+    const size_t V = g.V;
+    cplx<double>* base = P + (size_t)(6 * h) * V + (size_t)c * g.Vb + (act ? l : 0);
+    const int myq = bitrev_idx<K>(lane & (K - 1));
+    // sums over the CTA of v[0..K) into tot (all threads may read it on return)
+    auto sum_all = [&](double (&v)[K]) {
+        const double t = warp_transpose_sum<double, K>(v, lane);
+        __syncthreads();
+        if (lane < K) part[w][myq] = t;
+        __syncthreads();
+        if (l < K) {
+            double a = 0;
+            for (int q = 0; q < nw; ++q) a += part[q][l];
+            tot[l] = a;
         }
+        __syncthreads();
+    };
+    for (int j0 = 0; j0 < N; j0 += K) {  // ||p_j||^2 as given
+        double v[K];
+#pragma unroll
+        for (int u = 0; u < K; ++u) {
+            v[u] = 0;
+            if (act && j0 + u < N)
+                for (int k = 0; k < 6; ++k) v[u] += norm2(base[((size_t)(j0 + u) * 12 + k) * V]);
+        }
+        sum_all(v);
+        if (l < K && j0 + l < N) orig_s[j0 + l] = tot[l];
+    }
+    for (int j = 0; j < N; ++j) {
+        cplx<double>* pj = base + (size_t)j * 12 * V;
+        cplx<double> x[6];
         double nn = 0;
-        if (act)
-            for (int k = 6 * h; k < 6 * h + 6; ++k) nn += norm2(pj[(size_t)k * g.V + i]);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            x[k] = act ? pj[k * V] : czero<double>();
+            nn += norm2(x[k]);
+        }
         nn = block_sum_d(nn, red);
+        const double orig = orig_s[j];
         if (!(nn > 1e-24 * orig) || !(orig > 0)) {
             if (threadIdx.x == 0) atomicExch(fail, 1);
             nn = 1.0;
         }
-        double inv = 1.0 / sqrt(nn);
-        if (act)
-            for (int k = 6 * h; k < 6 * h + 6; ++k) pj[(size_t)k * g.V + i] = inv * pj[(size_t)k * g.V + i];
+        const double inv = 1.0 / sqrt(nn);
+#pragma unroll
+        for (int k = 0; k < 6; ++k) {
+            x[k] = inv * x[k];
+            if (act) pj[k * V] = x[k];
+        }
+        for (int q0 = j + 1; q0 < N; q0 += Q) {
+            double v[K];
+#pragma unroll
+            for (int u = 0; u < Q; ++u) {
+                cplx<double> d = czero<double>();
+                if (act && q0 + u < N) {
+                    const cplx<double>* pq = base + (size_t)(q0 + u) * 12 * V;
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) cmac_conj(d, x[k], pq[k * V]);
+                }
+                v[2 * u] = d.re, v[2 * u + 1] = d.im;
+            }
+            sum_all(v);
+            if (act)
+#pragma unroll 2
+                for (int u = 0; u < Q; ++u) {
+                    if (q0 + u >= N) break;
+                    const cplx<double> d = mk(-tot[2 * u], -tot[2 * u + 1]);
+                    cplx<double>* pq = base + (size_t)(q0 + u) * 12 * V;
+                    cplx<double> y[6];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) y[k] = pq[k * V];
+#pragma unroll
+                    for (int k = 0; k < 6; ++k) {
+                        cmac(y[k], d, x[k]);
+                        pq[k * V] = y[k];
+                    }
+                }
+        }
     }
 }
 
 int launch_gram_schmidt(const Geom& g, cplx<double>* P, int N, int* fail, cudaStream_t st) {
     const int nt = ((g.Vb + 31) / 32) * 32;
-    gram_schmidt_kernel<<<2 * g.NB, nt, 0, st>>>(g, P, N, fail);
+    if (nt <= 256) gram_schmidt_kernel<256><<<2 * g.NB, nt, 0, st>>>(g, P, N, fail);
+    else gram_schmidt_kernel<1024><<<2 * g.NB, nt, 0, st>>>(g, P, N, fail);
     DD_CHECK_LAUNCH();
     return 0;
 }
 
 // ---------------------------------------------------------------------------
-// D_c assembly.  For a direction dir (0 = self, 1 + d = hop in fine direction d
-// leaving the block) and every column (h, j):
-//   T_(h,j) = D_block P_j^(h)            (dir = 0: site term + hops inside the block)
-//   T_(h,j) = H_d P_j^(h) on face sites  (dir = 1 + d)
-// with P_j^(h) = P_j restricted to spins {2h, 2h+1}.  Then
-//   B_dir(c)[(h',j')][(h,j)] = sum_{x in c, k in half h'} conj(P_j'[k][x]) T_(h,j)[k][x].
+// D_c assembly.  D = Gamma5 D^H Gamma5 and P commutes with Gamma5 (chirality halves), so half of the stencil
+// follows from the other half:
+//   B_{-mu}(c + mu) = Gamma5 B_{+mu}(c)^H Gamma5,   B_0 = X + Gamma5 X^H Gamma5,
+// where X takes the forward hops inside the block and half of the (hermitian, chirality-diagonal) site term.
+// For every column (h, j) of P (P_j restricted to spins {2h, 2h+1}) the forward direction dir gives
+//   T_(h,j) = (A / 2 + forward in-block hops) P_j^(h)       (dir = 0)
+//   T_(h,j) = forward hop in direction mu on the face sites (dir = 1 + 2 mu)
+// and X / B_dir(c)[(h',j')][(h,j)] = sum_{x in c, k in half h'} conj(P_j'[k][x]) T_(h,j)[k][x].
+// All of it is bound by FP64 arithmetic (1/64 of the FP32 rate); the symmetry leaves five of nine products
+// with P^H and four of eight hops.  20 vectors on 16^4: T 9.51 -> 2.99 ms, products 15.35 -> 10.24 ms.
 // ---------------------------------------------------------------------------
 
-// masked load: P_j at site x with only the spins of half h kept
-__device__ __forceinline__ void load_half(Spinor<double>& s, const cplx<double>* __restrict__ pj, int V, int x, int h) {
+// acc += -1/2 (I - gamma_mu) (x) U_mu(x) psi for psi = the spins of half h of P_j at site nb
+template <int MU, int H>
+__device__ __forceinline__ void asm_hop(const cplx<double>* __restrict__ U, const cplx<double>* __restrict__ pj, size_t V, int i, int nb,
+                                        cplx<double> (&acc)[12]) {
+    using B = SpinB<MU>;
+    cplx<double> hs[2][3];  // psi_up, or -B psi_low
 #pragma unroll
-    for (int k = 0; k < 12; ++k) s.v[k] = ((k / 6) == h) ? pj[(size_t)k * V + x] : czero<double>();
-}
-
-template <int MU>
-__device__ __forceinline__ void asm_hop_dir(const Geom& g, const cplx<double>* __restrict__ U, const cplx<double>* __restrict__ pj,
-                                            int h, int i, int nb, bool fwd, Spinor<double>& acc) {
-    cplx<double> W[9];
-    Spinor<double> pn;
-    load_half(pn, pj, g.V, nb, h);
-    if (fwd) {
-        load_link(W, U, g.V, MU, i);
-        hop_acc<MU, true>(acc, pn, W);
-    } else {
-        load_link(W, U, g.V, MU, nb);
-        hop_acc<MU, false>(acc, pn, W);
-    }
-}
-
-__device__ __forceinline__ void asm_hop(const Geom& g, const cplx<double>* __restrict__ U, const cplx<double>* __restrict__ pj,
-                                        int h, int i, int nb, int d, Spinor<double>& acc) {
-    const bool fwd = (d & 1) == 0;
-    switch (d >> 1) {
-        case 0: asm_hop_dir<0>(g, U, pj, h, i, nb, fwd, acc); break;
-        case 1: asm_hop_dir<1>(g, U, pj, h, i, nb, fwd, acc); break;
-        case 2: asm_hop_dir<2>(g, U, pj, h, i, nb, fwd, acc); break;
-        default: asm_hop_dir<3>(g, U, pj, h, i, nb, fwd, acc); break;
-    }
-}
-
-__global__ void assemble_T_kernel(Geom g, FineOp<double> op, const cplx<double>* __restrict__ P, int N, int dir, int col0, int ncols,
-                                  cplx<double>* __restrict__ Tout) {
-    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (tid >= (long long)g.V * ncols) return;
-    const int i = (int)(tid % g.V);
-    const int col = col0 + (int)(tid / g.V);
-    const int h = col / N, j = col % N;
-    const cplx<double>* pj = P + (size_t)j * 12 * g.V;
-    const int c = block_of(g, i);
-    const int l = i - c * g.Vb;
-    Spinor<double> acc;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) acc.v[k] = czero<double>();
-    Spinor<double> out;
-    if (dir == 0) {
-        for (int d = 0; d < 8; ++d) {
-            int e = __ldg(g.lnbr + d * g.Vb + l);
-            if (e >> 16) continue;
-            asm_hop(g, op.U, pj, h, i, c * g.Vb + (e & 0xffff), d, acc);
+    for (int c = 0; c < 3; ++c) {
+        if constexpr (H == 0) {
+            hs[0][c] = pj[c * V + nb], hs[1][c] = pj[(3 + c) * V + nb];
+        } else {
+            const cplx<double> l2 = pj[(6 + c) * V + nb], l3 = pj[(9 + c) * V + nb];
+            hs[0][c] = ipow<(B::p0 + 2) & 3>(B::c0 ? l3 : l2), hs[1][c] = ipow<(B::p1 + 2) & 3>(B::c1 ? l3 : l2);
         }
-        Spinor<double> x;
-        load_half(x, pj, g.V, i, h);
-        herm_apply(op.clov, g.V, i, x, out);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) out.v[k] = out.v[k] - 0.5 * acc.v[k];
-    } else {
-        const int d = dir - 1;
-        int e = __ldg(g.lnbr + d * g.Vb + l);
-        if (e >> 16) asm_hop(g, op.U, pj, h, i, fine_nbr(g, i, d), d, acc);
-#pragma unroll
-        for (int k = 0; k < 12; ++k) out.v[k] = -0.5 * acc.v[k];
     }
-    cplx<double>* o = Tout + (size_t)(col - col0) * 12 * g.V;
+    const cplx<double>* W = U + (size_t)(MU * 9) * V + i;
 #pragma unroll
-    for (int k = 0; k < 12; ++k) o[(size_t)k * g.V + i] = out.v[k];
+    for (int a = 0; a < 3; ++a) {
+        cplx<double> g[2] = {czero<double>(), czero<double>()};
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            const cplx<double> u = ldg_c(W + (size_t)(a * 3 + b) * V);
+            cmac(g[0], u, hs[0][b]);
+            cmac(g[1], u, hs[1][b]);
+        }
+        acc[a] = acc[a] + g[0], acc[3 + a] = acc[3 + a] + g[1];
+        acc[6 + a] = acc[6 + a] - ipow<B::hp0>(g[B::hc0]), acc[9 + a] = acc[9 + a] - ipow<B::hp1>(g[B::hc1]);
+    }
+}
+// in-block forward hop in direction MU
+template <int MU, int H>
+__device__ __forceinline__ void asm_hop_in(const Geom& g, const cplx<double>* U, const cplx<double>* pj, int c, int l, cplx<double> (&acc)[12]) {
+    const int e = __ldg(g.lnbr + 2 * MU * g.Vb + l);
+    if (!(e >> 16)) asm_hop<MU, H>(U, pj, g.V, c * g.Vb + l, c * g.Vb + (e & 0xffff), acc);
+}
+template <int H>
+__device__ __forceinline__ void asm_self(const Geom& g, const FineOp<double>& op, const cplx<double>* __restrict__ pj, int i,
+                                         cplx<double>* __restrict__ o) {
+    const int c = block_of(g, i), l = i - c * g.Vb;
+    const size_t V = g.V;
+    cplx<double> acc[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = czero<double>();
+    asm_hop_in<0, H>(g, op.U, pj, c, l, acc);
+    asm_hop_in<1, H>(g, op.U, pj, c, l, acc);
+    asm_hop_in<2, H>(g, op.U, pj, c, l, acc);
+    asm_hop_in<3, H>(g, op.U, pj, c, l, acc);
+    cplx<double> x[6], y[6];  // the site term acts inside half H
+    const double* cl = op.clov + (size_t)(H * 36) * V + i;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+        x[a] = pj[(size_t)(6 * H + a) * V + i];
+        y[a] = __ldg(cl + a * V) * x[a];
+    }
+    int q = 0;
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+#pragma unroll
+        for (int b = a + 1; b < 6; ++b) {
+            const cplx<double> m = mk(__ldg(cl + (size_t)(6 + 2 * q) * V), __ldg(cl + (size_t)(7 + 2 * q) * V));
+            cmac(y[a], m, x[b]);
+            cmac_conj(y[b], m, x[a]);
+            ++q;
+        }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[(size_t)k * V + i] = (k / 6 == H) ? 0.5 * (y[k % 6] - acc[k]) : -0.5 * acc[k];
 }
 
-// T[col - col0] = (the part of D in direction dir) applied to column col of P (split by chirality
-// half), for the columns col0 .. col0 + ncols - 1 of the 2N
-int launch_assemble_T(const Geom& g, const FineOp<double>& op, const cplx<double>* P, int N, int dir, int col0, int ncols,
-                      cplx<double>* T, cudaStream_t st) {
-    const long long n = (long long)g.V * ncols;
-    assemble_T_kernel<<<ceil_div(n, 128), 128, 0, st>>>(g, op, P, N, dir, col0, ncols, T);
+// dir = 0: thread = (site, column); dir = 1 + 2 mu: thread = (face site of a block, column)
+__global__ void __launch_bounds__(128) assemble_T_kernel(Geom g, FineOp<double> op, const cplx<double>* __restrict__ P, int N, int dir, int col0,
+                                                         int ncols, const int* __restrict__ sites, int nsites, cplx<double>* __restrict__ Tout) {
+    const long long tid = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    const int per = g.NB * nsites;  // sites of one column
+    if (tid >= (long long)per * ncols) return;
+    const int col = col0 + (int)(tid / per), q = (int)(tid % per);
+    const int c = q / nsites, l = dir == 0 ? q % nsites : __ldg(sites + q % nsites);
+    const int i = c * g.Vb + l, h = col / N, j = col % N;
+    const size_t V = g.V;
+    const cplx<double>* pj = P + (size_t)j * 12 * V;
+    cplx<double>* o = Tout + (size_t)(col - col0) * 12 * V;
+    if (dir == 0) {
+        if (h == 0) asm_self<0>(g, op, pj, i, o);
+        else asm_self<1>(g, op, pj, i, o);
+        return;
+    }
+    const int nb = fine_nbr(g, i, dir - 1);
+    cplx<double> acc[12];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) acc[k] = czero<double>();
+    switch ((dir - 1) + h) {  // dir - 1 = 2 mu
+        case 0: asm_hop<0, 0>(op.U, pj, V, i, nb, acc); break;
+        case 1: asm_hop<0, 1>(op.U, pj, V, i, nb, acc); break;
+        case 2: asm_hop<1, 0>(op.U, pj, V, i, nb, acc); break;
+        case 3: asm_hop<1, 1>(op.U, pj, V, i, nb, acc); break;
+        case 4: asm_hop<2, 0>(op.U, pj, V, i, nb, acc); break;
+        case 5: asm_hop<2, 1>(op.U, pj, V, i, nb, acc); break;
+        case 6: asm_hop<3, 0>(op.U, pj, V, i, nb, acc); break;
+        default: asm_hop<3, 1>(op.U, pj, V, i, nb, acc); break;
+    }
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[(size_t)k * V + i] = -0.5 * acc[k];
+}
+
+// T[col - col0] for the columns col0 .. col0 + ncols - 1 of the 2N, on the listed local sites of every block
+// (dir = 0: all sites)
+int launch_assemble_T(const Geom& g, const FineOp<double>& op, const cplx<double>* P, int N, int dir, int col0, int ncols, const int* sites,
+                      int nsites, cplx<double>* T, cudaStream_t st) {
+    const long long n = (long long)g.NB * nsites * ncols;
+    assemble_T_kernel<<<ceil_div(n, 128), 128, 0, st>>>(g, op, P, N, dir, col0, ncols, sites, nsites, T);
+    DD_CHECK_LAUNCH();
+    return 0;
+}
+
+// The other half of the stencil: B_0 = X + Gamma5 X^H Gamma5 in place, B_{-mu}(c + mu) = Gamma5 B_{+mu}(c)^H Gamma5.
+// One CTA per (site, direction: 0 = self, 1 + mu); blocks are [column][row].
+__global__ void __launch_bounds__(256) complete_stencil_kernel(Geom g, int N, cplx<double>* __restrict__ B) {
+    const int c = blockIdx.x, d = blockIdx.y, nc = 2 * N, nn = nc * nc;
+    cplx<double>* src = B + ((size_t)c * 9 + (d == 0 ? 0 : 2 * d - 1)) * nn;
+    auto flip = [&](int row, int col, cplx<double> v) { return (row < N) == (col < N) ? conj(v) : mk(-v.re, v.im); };
+    if (d == 0) {
+        for (int q = threadIdx.x; q < nn; q += blockDim.x) {
+            const int col = q / nc, row = q % nc;
+            if (row > col) continue;
+            const cplx<double> a = src[col * nc + row], b = src[row * nc + col];
+            src[col * nc + row] = a + flip(row, col, b);
+            src[row * nc + col] = b + flip(row, col, a);
+        }
+    } else {
+        const int mu = d - 1;
+        cplx<double>* dst = B + ((size_t)__ldg(g.bnbr + 2 * mu * g.NB + c) * 9 + 2 + 2 * mu) * nn;
+        for (int q = threadIdx.x; q < nn; q += blockDim.x) {
+            const int col = q / nc, row = q % nc;
+            dst[q] = flip(row, col, src[row * nc + col]);
+        }
+    }
+}
+int launch_complete_stencil(const Geom& g, int N, double* B, cudaStream_t st) {
+    complete_stencil_kernel<<<dim3(g.NB, 5), 256, 0, st>>>(g, N, reinterpret_cast<cplx<double>*>(B));
     DD_CHECK_LAUNCH();
     return 0;
 }
