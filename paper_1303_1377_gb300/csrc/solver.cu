@@ -260,6 +260,7 @@ struct ddamg_handle {
     CoarseTC tc{};
     int* d_flag = nullptr;
     int* d_tc_err = nullptr;  // half mode: set by a coarse-stencil kernel whose bulk copy did not complete
+    int* h_tc_err = nullptr;  // its pinned copy
     // workspaces
     Scratch ws_fine[6], ws_coarse[8], ws_io[3], ws_outer[5];
     Scratch ws_rmax;  // per right-hand-side field maxima of the tensor-core restriction
@@ -1490,13 +1491,15 @@ static int solve_T(ddamg_handle* h, const cplx<double>* b, cplx<double>* x, int 
 }
 
 // half mode: a coarse-stencil kernel whose bulk copy of the site matrix never completed sets a
-// device flag (the kernel gives up after a bounded wait instead of hanging); report it as a CUDA error
+// device flag (the kernel gives up after a bounded wait instead of hanging); it is reported as a CUDA
+// error.  The flag is fetched into pinned memory (tc_fetch) ahead of the synchronisation that ends the call anyway
+// (finish_out), and read after it (tc_check).
+static int tc_fetch(ddamg_handle* h) {
+    if (h->d_tc_err) DD_CUDA(cudaMemcpyAsync(h->h_tc_err, h->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
+    return 0;
+}
 static int tc_check(ddamg_handle* h) {
-    if (!h->d_tc_err) return 0;
-    int f = 0;
-    DD_CUDA(cudaMemcpyAsync(&f, h->d_tc_err, sizeof(int), cudaMemcpyDeviceToHost, h->stream));
-    DD_CUDA(cudaStreamSynchronize(h->stream));
-    if (f) {
+    if (h->d_tc_err && *h->h_tc_err) {
         set_error("coarse stencil: a bulk copy of the site matrix did not complete within the kernel's wait limit");
         return DDAMG_ERR_CUDA;
     }
@@ -1629,7 +1632,12 @@ static int create(const ddamg_lattice* lat, const double* U, double m0, double c
             (rc = dalloc_n(&h->P16, V * 12 * N)))
             return fail(rc);
         if ((rc = dalloc_n(&h->d_tc_err, 1))) return fail(rc);
-        if (cudaMemset(h->d_tc_err, 0, sizeof(int)) != cudaSuccess) return fail(DDAMG_ERR_CUDA);
+        if (cudaMemset(h->d_tc_err, 0, sizeof(int)) != cudaSuccess || cudaMallocHost(&h->h_tc_err, sizeof(int)) != cudaSuccess) {
+            (void)cudaGetLastError();
+            set_error("half mode: the error flag could not be set up");
+            return fail(DDAMG_ERR_CUDA);
+        }
+        *h->h_tc_err = 0;
         h->tc = CoarseTC{h->Bh, h->Dh, h->d_bnbr, h->NB, (int)nc, Mt, Kta, Kth, Ktd, h->d_tc_err};
         const size_t cw16 = h->g.blk44 ? 10 : 9;  // 16-byte words of a site term (clover_to_aos16)
         if (p.smoother_fp16 &&
@@ -1854,6 +1862,7 @@ static int solve_common(ddamg_handle* h, const double* b, double* z, int nrhs, d
              : h->p.outer == DDAMG_OUTER_REFINE ? solve_T<float, float>(h, bi, xi, nrhs, tol, x0_zero, R, nullptr, 0, dl)
                                                 : solve_T<float, dwf>(h, bi, xi, nrhs, tol, x0_zero, R, nullptr, 0, dl);
     if (rc) return rc;
+    DD_TRY(tc_fetch(h));
     DD_TRY(fine_out<double>(h, xi, z, nrhs));
     DD_TRY(tc_check(h));
     double secs = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
@@ -2105,6 +2114,7 @@ static int restrict_T(ddamg_handle* h, const double* in, double* out, int n_rhs)
     cplx<T>* o = a + fld * n_rhs;
     DD_TRY(fine_in<T>(h, in, n_rhs, h->ws_io[0], a));
     DD_TRY(restrict_<T>(h, a, o, n_rhs));
+    DD_TRY(tc_fetch(h));
     DD_TRY(coarse_out<T>(h, o, out, n_rhs));
     return tc_check(h);
 }
@@ -2149,6 +2159,7 @@ static int apply_Dc_T(ddamg_handle* h, const double* in, double* out, int n_rhs)
         Prof pr(h, PF_COARSE, (double)h->NB * 9 * h->nc * h->nc * sizeof(cplx<T>));
         DD_TRY(c_full<T>(h, a, o, n_rhs));
     }
+    DD_TRY(tc_fetch(h));
     DD_TRY(coarse_out<T>(h, o, out, n_rhs));
     return tc_check(h);
 }
@@ -2237,6 +2248,7 @@ static int coarse_solve_T(ddamg_handle* h, const double* in, double* out, int n_
     DD_TRY(coarse_in<T>(h, in, n_rhs, a));
     h->coarse_iters = 0;
     DD_TRY(coarse_solve<T>(h, a, o, n_rhs, fixed));
+    DD_TRY(tc_fetch(h));
     DD_TRY(coarse_out<T>(h, o, out, n_rhs));
     return tc_check(h);
 }
@@ -2408,6 +2420,7 @@ int ddamg_destroy(ddamg_handle* h) {
     dfree(h->P16);
     dfree(h->d_flag);
     dfree(h->d_tc_err);
+    if (h->h_tc_err) cudaFreeHost(h->h_tc_err);
     for (auto& s : h->ws_fine) s.release();
     for (auto& s : h->ws_coarse) s.release();
     for (auto& s : h->ws_io) s.release();

@@ -237,6 +237,12 @@ def _ptr(a):
     return C.c_void_p(a.ctypes.data)
 
 
+def _ptr_new(a):
+    """Pointer of an output that this module has just allocated beside an input already passed to _ptr: the wait
+    there covers every use that torch's stream still had of the memory."""
+    return C.c_void_p(a.data_ptr() if _is_torch(a) else a.ctypes.data)
+
+
 def _host(a, dtype):
     if _is_torch(a):
         return a
@@ -386,7 +392,7 @@ class Solver:
         x = _host(x, np.complex128)
         nr = int(x.shape[0])
         out = _empty_like(x, (nr,) + tuple(out_shape), np.complex128)
-        _check(fn(self.h, _ptr(x), _ptr(out), nr, *extra), fn.__name__)
+        _check(fn(self.h, _ptr(x), _ptr_new(out), nr, *extra), fn.__name__)
         return out
 
     def ml_apply_sap1(self, x, nu: int):
@@ -469,7 +475,7 @@ class Solver:
         x = _host(x, dtype)
         nr = 1 if x.ndim == 3 else int(x.shape[0])
         out = _empty_like(x, x.shape, dtype)
-        _check(fn(self.h, _ptr(x), _ptr(out), nr, *extra), fn.__name__)
+        _check(fn(self.h, _ptr(x), _ptr_new(out), nr, *extra), fn.__name__)
         return out
 
     def apply_D(self, x):
@@ -483,7 +489,7 @@ class Solver:
         x = _host(x, np.complex64)
         nr = 1 if x.ndim == 3 else int(x.shape[0])
         out = _empty_like(x, x.shape, np.complex128)
-        _check(lib.ddamg_apply_D_mixed(self.h, _ptr(x), _ptr(out), nr), "ddamg_apply_D_mixed")
+        _check(lib.ddamg_apply_D_mixed(self.h, _ptr(x), _ptr_new(out), nr), "ddamg_apply_D_mixed")
         return out
 
     def apply_sap(self, x, nu: int):
@@ -496,21 +502,21 @@ class Solver:
         x = _host(x, np.complex128)
         nr = 1 if x.ndim == 3 else int(x.shape[0])
         out = _empty_like(x, (nr, self.n_coarse, self.coarse_dof), np.complex128)
-        _check(lib.ddamg_restrict(self.h, _ptr(x), _ptr(out), nr), "ddamg_restrict")
+        _check(lib.ddamg_restrict(self.h, _ptr(x), _ptr_new(out), nr), "ddamg_restrict")
         return out[0] if x.ndim == 3 else out
 
     def prolong(self, e):
         e = _host(e, np.complex128)
         nr = 1 if e.ndim == 2 else int(e.shape[0])
         out = _empty_like(e, (nr, self.V, 4, 3), np.complex128)
-        _check(lib.ddamg_prolong(self.h, _ptr(e), _ptr(out), nr), "ddamg_prolong")
+        _check(lib.ddamg_prolong(self.h, _ptr(e), _ptr_new(out), nr), "ddamg_prolong")
         return out[0] if e.ndim == 2 else out
 
     def _coarse_op(self, fn, e, *extra):
         e = _host(e, np.complex128)
         nr = 1 if e.ndim == 2 else int(e.shape[0])
         out = _empty_like(e, e.shape, np.complex128)
-        _check(fn(self.h, _ptr(e), _ptr(out), nr, *extra), fn.__name__)
+        _check(fn(self.h, _ptr(e), _ptr_new(out), nr, *extra), fn.__name__)
         return out
 
     def apply_Dc(self, e):
