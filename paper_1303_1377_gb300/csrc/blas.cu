@@ -145,15 +145,34 @@ int convert(const Ti* in, To* out, size_t n, cudaStream_t st) {
 }
 
 // ABI lexicographic field [nrhs][V][ncomp] <-> internal [nrhs][ncomp][V];  lex_of[i] = lexicographic site of internal i
-template <typename To, typename Ti>
-__global__ void to_internal_kernel(const cplx<Ti>* __restrict__ in, cplx<To>* __restrict__ out, const int* __restrict__ lex_of, int V,
-                                   int ncomp, int nrhs) {
+// MAX: also rmax[r] = bits of max |Re|, |Im| of right-hand side r as stored (non-negative floats order like their
+// bits).  V is a multiple of 256, so a CTA's 256 sites belong to one right-hand side.
+template <typename To, typename Ti, bool MAX>
+__global__ void __launch_bounds__(256) to_internal_kernel(const cplx<Ti>* __restrict__ in, cplx<To>* __restrict__ out,
+                                                          const int* __restrict__ lex_of, int V, int ncomp, int nrhs, int* __restrict__ rmax) {
     const size_t tot = (size_t)V * nrhs;
     for (size_t q = (size_t)blockIdx.x * blockDim.x + threadIdx.x; q < tot; q += (size_t)gridDim.x * blockDim.x) {
         int r = (int)(q / V), i = (int)(q % V);
         const cplx<Ti>* src = in + ((size_t)r * V + lex_of[i]) * ncomp;
         cplx<To>* dst = out + (size_t)r * ncomp * V + i;
-        for (int k = 0; k < ncomp; ++k) dst[(size_t)k * V] = ccast<To>(src[k]);
+        float m = 0.f;
+        for (int k = 0; k < ncomp; ++k) {
+            const cplx<To> v = ccast<To>(src[k]);
+            dst[(size_t)k * V] = v;
+            if (MAX) m = fmaxf(m, fmaxf(fabsf((float)v.re), fabsf((float)v.im)));
+        }
+        if constexpr (MAX) {
+            __shared__ float ms[8];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
+            if ((threadIdx.x & 31) == 0) ms[threadIdx.x >> 5] = m;
+            __syncthreads();
+            if (threadIdx.x == 0) {
+                for (int w = 1; w < 8; ++w) m = fmaxf(m, ms[w]);
+                atomicMax(rmax + r, __float_as_int(m));
+            }
+            __syncthreads();
+        }
     }
 }
 
@@ -191,7 +210,16 @@ template <typename To, typename Ti>
 int to_internal(const cplx<Ti>* in, cplx<To>* out, const int* lex_of, int V, int ncomp, int nrhs, cudaStream_t st) {
     int blocks = ceil_div((long long)V * nrhs, 256);
     if (blocks > 152 * 32) blocks = 152 * 32;
-    to_internal_kernel<To, Ti><<<blocks, 256, 0, st>>>(in, out, lex_of, V, ncomp, nrhs);
+    to_internal_kernel<To, Ti, false><<<blocks, 256, 0, st>>>(in, out, lex_of, V, ncomp, nrhs, nullptr);
+    DD_CHECK_LAUNCH();
+    return 0;
+}
+int to_internal_max(const cplx<double>* in, cplx<float>* out, const int* lex_of, int V, int ncomp, int nrhs, int* rmax, cudaStream_t st) {
+    if (V % 256) return DDAMG_ERR_INVALID_ARG;
+    int blocks = ceil_div((long long)V * nrhs, 256);
+    if (blocks > 152 * 32) blocks = 152 * 32;
+    DD_CUDA(cudaMemsetAsync(rmax, 0, sizeof(int) * nrhs, st));
+    to_internal_kernel<float, double, true><<<blocks, 256, 0, st>>>(in, out, lex_of, V, ncomp, nrhs, rmax);
     DD_CHECK_LAUNCH();
     return 0;
 }

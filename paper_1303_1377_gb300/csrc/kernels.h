@@ -85,9 +85,9 @@ template <typename T, typename Tp>
 int launch_prolong(const Geom& g, const cplx<Tp>* P, int N, const cplx<T>* in, cplx<T>* out, int nrhs, cudaStream_t st);
 // half-precision V-cycle: restriction as FP16 tensor-core products (needs Vb % 16 == 0, N % 4 == 0, N <= 32)
 bool restrict_tc_supported(const Geom& g, int N);
-// rmax: nrhs ints of device scratch (the field maxima)
+// rmax: nrhs ints of device scratch for the field maxima (bits of max |Re|, |Im|); have_max: it holds them already
 int launch_restrict_tc(const Geom& g, const cplx<__half>* P, int N, const cplx<float>* in, cplx<float>* out, int nrhs, int* rmax,
-                       cudaStream_t st);
+                       bool have_max, cudaStream_t st);
 // half-precision V-cycle: prolongation as FP16 tensor-core products (needs Vb % 16 == 0, N <= 32)
 bool prolong_tc_supported(const Geom& g, int N);
 int launch_prolong_tc(const Geom& g, const cplx<__half>* P, int N, const cplx<float>* in, cplx<float>* out, int nrhs, cudaStream_t st);

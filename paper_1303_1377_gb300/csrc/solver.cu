@@ -621,7 +621,7 @@ static int sap(ddamg_handle* h, const cplx<T>* b, cplx<T>* z, int nrhs, int nu) 
 }
 
 template <typename T>
-static int restrict_(ddamg_handle* h, const cplx<T>* in, cplx<T>* out, int nrhs) {
+static int restrict_(ddamg_handle* h, const cplx<T>* in, cplx<T>* out, int nrhs, bool have_max = false) {
     Level<T> L = level<T>(h);
     const double pb = h->half() ? 2.0 : sizeof(T);
     Prof pr(h, PF_RESTRICT, (double)h->V * (12.0 * h->N * 2 * pb + 12.0 * nrhs * 2 * sizeof(T)));
@@ -629,7 +629,7 @@ static int restrict_(ddamg_handle* h, const cplx<T>* in, cplx<T>* out, int nrhs)
         if (restrict_tc_supported(h->g, h->N)) {
             DD_TRY(h->ws_rmax.ensure(sizeof(int) * nrhs));
             return launch_restrict_tc(h->g, h->P16, h->N, reinterpret_cast<const cplx<float>*>(in), reinterpret_cast<cplx<float>*>(out),
-                                      nrhs, h->ws_rmax.as<int>(), h->stream);
+                                      nrhs, h->ws_rmax.as<int>(), have_max, h->stream);
         }
         return launch_restrict<float, __half>(h->g, h->P16, h->N, reinterpret_cast<const cplx<float>*>(in),
                                               reinterpret_cast<cplx<float>*>(out), nrhs, h->stream);
@@ -2112,8 +2112,19 @@ static int restrict_T(ddamg_handle* h, const double* in, double* out, int n_rhs)
     DD_TRY(h->ws_fine[4].ensure(sizeof(cplx<T>) * (fld + cn) * n_rhs));
     cplx<T>* a = h->ws_fine[4].as<cplx<T>>();
     cplx<T>* o = a + fld * n_rhs;
-    DD_TRY(fine_in<T>(h, in, n_rhs, h->ws_io[0], a));
-    DD_TRY(restrict_<T>(h, a, o, n_rhs));
+    bool have_max = false;
+    if constexpr (std::is_same<T, float>::value) {
+        if (h->half() && restrict_tc_supported(h->g, h->N) && h->V % 256 == 0) {
+            // the FP16 restriction scales by the fields' maxima: found while the fields are brought in
+            const void* dv;
+            DD_TRY(h->ws_rmax.ensure(sizeof(int) * n_rhs));
+            DD_TRY(stage_in(h, h->ws_io[0], in, sizeof(cplx<double>) * fld * n_rhs, &dv));
+            DD_TRY(to_internal_max(reinterpret_cast<const cplx<double>*>(dv), a, h->d_lex_of, h->V, 12, n_rhs, h->ws_rmax.as<int>(), h->stream));
+            have_max = true;
+        }
+    }
+    if (!have_max) DD_TRY(fine_in<T>(h, in, n_rhs, h->ws_io[0], a));
+    DD_TRY(restrict_<T>(h, a, o, n_rhs, have_max));
     DD_TRY(tc_fetch(h));
     DD_TRY(coarse_out<T>(h, o, out, n_rhs));
     return tc_check(h);

@@ -138,8 +138,12 @@ __global__ void __launch_bounds__(kProTCWarps * 32) prolong_tc_kernel(Geom g, co
 // ---------------------------------------------------------------------------
 constexpr int kResTCWarps = 8;
 
+// Bound by the latency of the loads of P and of the fields.  Two CTAs per SM fit either way (shared memory would
+// allow three); asking for no more lets a thread keep two k-tiles of loads in flight in 128 registers instead of
+// the 84 the compiler chose: 12 fields, N = 20, with the pass for the maxima: 24^4 390 -> 221 us, 32x16^3 164 ->
+// 96 us.  Three or four CTAs (80, 64 registers) 260 and 363 us, one or four k-tiles 225 and 240 us (24^4).
 template <int NTN>  // n-tiles over (j, re/im): N = 4 NTN test vectors
-__global__ void __launch_bounds__(kResTCWarps * 32) restrict_tc_kernel(Geom g, const __half2* __restrict__ P, int N,
+__global__ void __launch_bounds__(kResTCWarps * 32, 2) restrict_tc_kernel(Geom g, const __half2* __restrict__ P, int N,
                                                                         const cplx<float>* __restrict__ in, cplx<float>* __restrict__ out,
                                                                         int nrhs, int r0, const int* __restrict__ rmax) {
     constexpr int MT = 2;  // 16 right-hand sides per launch group
@@ -250,15 +254,17 @@ __global__ void field_absmax_kernel(const float4* __restrict__ in, size_t n4, in
 bool restrict_tc_supported(const Geom& g, int N) { return g.Vb % 16 == 0 && N % 4 == 0 && N <= 32; }
 
 int launch_restrict_tc(const Geom& g, const cplx<__half>* P, int N, const cplx<float>* in, cplx<float>* out, int nrhs, int* rmax,
-                       cudaStream_t st) {
+                       bool have_max, cudaStream_t st) {
     const __half2* P2 = reinterpret_cast<const __half2*>(P);
     const int NTN = N / 4;
     const size_t sm = (size_t)kResTCWarps * 32 * 2 * NTN * 4 * sizeof(float);
     const size_t n4 = (size_t)12 * g.V / 2;  // float4 = two complex numbers; 12 V is even
-    DD_CUDA(cudaMemsetAsync(rmax, 0, sizeof(int) * nrhs, st));
-    const int bx = (int)std::min<size_t>((n4 + 255) / 256, (size_t)std::max(1, 152 * 8 / nrhs));
-    field_absmax_kernel<<<dim3(bx, nrhs), 256, 0, st>>>(reinterpret_cast<const float4*>(in), n4, rmax);
-    DD_CHECK_LAUNCH();
+    if (!have_max) {
+        DD_CUDA(cudaMemsetAsync(rmax, 0, sizeof(int) * nrhs, st));
+        const int bx = (int)std::min<size_t>((n4 + 255) / 256, (size_t)std::max(1, 152 * 8 / nrhs));
+        field_absmax_kernel<<<dim3(bx, nrhs), 256, 0, st>>>(reinterpret_cast<const float4*>(in), n4, rmax);
+        DD_CHECK_LAUNCH();
+    }
     for (int r0 = 0; r0 < nrhs; r0 += 16) {
         switch (NTN) {
 #define DD_RES_TC(n)                                                                                                   \

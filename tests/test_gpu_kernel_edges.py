@@ -141,3 +141,25 @@ def test_coarse_gmres_steps_by_vector_length(dims, block, n_vec, nrhs, steps):
             out[prec] = s.coarse_solve(e, steps)
     for r in range(nrhs):
         assert np.max(np.abs(out["SINGLE"][r] - out["DOUBLE"][r])) < 1e-6 * np.max(np.abs(out["DOUBLE"][r]))
+
+
+@pytest.mark.parametrize("dims,n_vec,nrhs", [((8, 8, 8, 8), 4, 1), ((8, 8, 16, 8), 12, 17), ((16, 8, 8, 24), 20, 5)])
+def test_half_restriction_of_fields_of_very_different_size(dims, n_vec, nrhs):
+    """P^H on half-precision handles scales every field by its own maximum: fields from 1e-30 to 1e30 and a zero
+    field, each to the stated 4e-3 of its own result's maximum."""
+    from oracle.aggregation import Aggregation
+    from oracle.dirac import DiracOperator
+    from paper_1303_1377_gb300 import ddamg
+
+    s, U = _solver(dims, n_vec=n_vec, precision=ddamg.PREC_HALF)
+    v = synth.random_test_vectors(dims, n_vec, seed=71)
+    x = synth.gaussian_spinors(dims, nrhs, seed=72)
+    x *= 10.0 ** np.linspace(-30, 30, nrhs)[:, None, None, None]
+    x[nrhs // 2] = 0
+    with s:
+        s.setup_from_vectors(v)
+        got = s.restrict(x)
+    agg = Aggregation(DiracOperator(U, dims, -0.4, 1.0).lat, (4, 4, 4, 4), v)
+    for r in range(nrhs):
+        ref = agg.restrict(x[r])
+        assert np.max(np.abs(got[r] - ref)) <= 4e-3 * np.max(np.abs(ref))
