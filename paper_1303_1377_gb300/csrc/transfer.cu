@@ -49,7 +49,7 @@ __device__ __forceinline__ T warp_transpose_sum(T (&v)[K], int lane) {
     return s;
 }
 
-template <typename T, typename Tp, int R>
+template <typename T, typename Tp, int R, bool SPLIT>
 __global__ void restrict_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, const cplx<T>* __restrict__ in,
                                 cplx<T>* __restrict__ out, int r0, int ngroups) {
     // accumulation in the V-cycle precision T (FP64 arithmetic is a small fraction of FP32 on GB300)
@@ -70,8 +70,10 @@ __global__ void restrict_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, c
     }
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int myq = bitrev_idx<K>(lane & (K - 1));
+    // SPLIT: gridDim.y CTAs per aggregate, each with its part of the test vectors
+    const int j0 = SPLIT ? blockIdx.y * N / gridDim.y : 0, j1 = SPLIT ? (blockIdx.y + 1) * N / gridDim.y : N;
 #pragma unroll 2
-    for (int j = 0; j < N; ++j) {
+    for (int j = j0; j < j1; ++j) {
         T v[K];
 #pragma unroll
         for (int q = 0; q < K; ++q) v[q] = 0;
@@ -93,7 +95,7 @@ __global__ void restrict_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, c
         if (lane < K) red[((size_t)w * N + j) * K + myq] = s;
     }
     __syncthreads();
-    for (int q = threadIdx.x; q < K * N; q += blockDim.x) {
+    for (int q = K * j0 + threadIdx.x; q < K * j1; q += blockDim.x) {
         T s = 0;
         for (int ww = 0; ww < nw; ++ww) s += red[(size_t)ww * K * N + q];
         const int j = q / K, t = q % K;
@@ -103,14 +105,30 @@ __global__ void restrict_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, c
     }
 }
 
+// Few aggregates: several CTAs share one, each with a part of the test vectors (restriction) or of the twelve
+// components (prolongation); a CTA reads its part of P one vector after the other and waits for each.  Up to 1216
+// CTAs (eight of 256 threads per SM).  N = 20, one field: FP32 16^4 (256 aggregates) restriction 78 -> 37 us,
+// prolongation 52 -> 32 us; 8^4 31 -> 10 and 19 -> 10 us; FP64 16^4 231 -> 203 and 131 -> 113 us.  The restriction of
+// two fields per CTA is not split: with the vector range at run time the compiler keeps fewer loads in flight
+// (24^4, 12 fields: 640 -> 1630 us).
+static unsigned transfer_split(long long nblk, int parts) {
+    unsigned s = 1;
+    while (s < 4 && (int)(2 * s) <= parts && nblk * s * 2 <= 4 * 304) s *= 2;
+    return s;
+}
+
 template <typename T, typename Tp, int R>
 static int launch_restrict_r(const Geom& g, const cplx<Tp>* P, int N, const cplx<T>* in, cplx<T>* out, int r0, int ngroups,
                              cudaStream_t st) {
     const int nt = ((g.Vb + 31) / 32) * 32;
     const long long nblk = (long long)g.NB * ngroups;
     size_t sm = (size_t)(nt / 32) * 4 * R * N * sizeof(T);
-    if (sm > 48 * 1024) cudaFuncSetAttribute(restrict_kernel<T, Tp, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
-    restrict_kernel<T, Tp, R><<<(unsigned)nblk, nt, sm, st>>>(g, P, N, in, out, r0, ngroups);
+    const unsigned split = R == 1 ? transfer_split(nblk, N) : 1;
+    auto* kernel = restrict_kernel<T, Tp, R, false>;
+    if constexpr (R == 1)
+        if (split > 1) kernel = restrict_kernel<T, Tp, R, true>;
+    if (sm > 48 * 1024) cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sm);
+    kernel<<<dim3((unsigned)nblk, split), nt, sm, st>>>(g, P, N, in, out, r0, ngroups);
     DD_CHECK_LAUNCH();
     return 0;
 }
@@ -131,7 +149,8 @@ int launch_restrict(const Geom& g, const cplx<Tp>* P, int N, const cplx<T>* in, 
 // prolongation out[r][k][x] = sum_j P_j[k][x] in[r][c(x)][h(k)*N + j]
 // CTA = (block c, group of R right-hand sides); every P_j entry loaded once serves R.
 // ---------------------------------------------------------------------------
-template <typename T, typename Tp, int R>
+// KC components per CTA: blockIdx.y * KC ...
+template <typename T, typename Tp, int R, int KC>
 __global__ void prolong_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, const cplx<T>* __restrict__ in,
                                cplx<T>* __restrict__ out, int r0, int ngroups) {
     extern __shared__ unsigned char smem_raw[];
@@ -146,11 +165,13 @@ __global__ void prolong_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, co
     const int l = threadIdx.x;
     if (l >= g.Vb) return;
     const int i = c * g.Vb + l;
-    cplx<T> acc[R][12];
+    const int k0 = blockIdx.y * KC;
+    cplx<T> acc[R][KC];
 #pragma unroll
     for (int u = 0; u < R; ++u)
 #pragma unroll
-        for (int k = 0; k < 12; ++k) acc[u][k] = czero<T>();
+        for (int k = 0; k < KC; ++k) acc[u][k] = czero<T>();
+#pragma unroll(R == 1 && (KC < 12 || sizeof(T) == 8) ? 4 : 1)
     for (int j = 0; j < N; ++j) {
         const cplx<Tp>* pj = P + (size_t)j * 12 * g.V;
         cplx<T> e0[R], e1[R];
@@ -160,17 +181,17 @@ __global__ void prolong_kernel(Geom g, const cplx<Tp>* __restrict__ P, int N, co
             e1[u] = e[u * 2 * N + N + j];
         }
 #pragma unroll
-        for (int k = 0; k < 12; ++k) {
-            const cplx<T> p = ccast<T>(pj[(size_t)k * g.V + i]);
+        for (int k = 0; k < KC; ++k) {
+            const cplx<T> p = ccast<T>(pj[(size_t)(k0 + k) * g.V + i]);
 #pragma unroll
-            for (int u = 0; u < R; ++u) cmac(acc[u][k], p, k < 6 ? e0[u] : e1[u]);
+            for (int u = 0; u < R; ++u) cmac(acc[u][k], p, k0 + k < 6 ? e0[u] : e1[u]);
         }
     }
 #pragma unroll
     for (int u = 0; u < R; ++u) {
         cplx<T>* o = out + (size_t)(rb + u) * 12 * g.V;
 #pragma unroll
-        for (int k = 0; k < 12; ++k) o[(size_t)k * g.V + i] = acc[u][k];
+        for (int k = 0; k < KC; ++k) o[(size_t)(k0 + k) * g.V + i] = acc[u][k];
     }
 }
 
@@ -179,7 +200,11 @@ static int launch_prolong_r(const Geom& g, const cplx<Tp>* P, int N, const cplx<
                             cudaStream_t st) {
     const int nt = ((g.Vb + 31) / 32) * 32;
     const long long nblk = (long long)g.NB * ngroups;
-    prolong_kernel<T, Tp, R><<<(unsigned)nblk, nt, 2 * N * R * sizeof(cplx<T>), st>>>(g, P, N, in, out, r0, ngroups);
+    const size_t sm = 2 * N * R * sizeof(cplx<T>);
+    const unsigned split = transfer_split(nblk, 12);
+    if (split == 4) prolong_kernel<T, Tp, R, 3><<<dim3((unsigned)nblk, 4), nt, sm, st>>>(g, P, N, in, out, r0, ngroups);
+    else if (split == 2) prolong_kernel<T, Tp, R, 6><<<dim3((unsigned)nblk, 2), nt, sm, st>>>(g, P, N, in, out, r0, ngroups);
+    else prolong_kernel<T, Tp, R, 12><<<(unsigned)nblk, nt, sm, st>>>(g, P, N, in, out, r0, ngroups);
     DD_CHECK_LAUNCH();
     return 0;
 }

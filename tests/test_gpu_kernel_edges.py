@@ -163,3 +163,26 @@ def test_half_restriction_of_fields_of_very_different_size(dims, n_vec, nrhs):
     for r in range(nrhs):
         ref = agg.restrict(x[r])
         assert np.max(np.abs(got[r] - ref)) <= 4e-3 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("prec,tol", [("DOUBLE", 1e-13), ("SINGLE", 1e-6)])
+@pytest.mark.parametrize("dims,block,n_vec,nrhs", [((4, 4, 4, 4), (2, 2, 2, 2), 1, 1), ((8, 8, 8, 8), (4, 4, 4, 4), 3, 3),
+                                                   ((16, 8, 8, 8), (2, 2, 4, 4), 7, 1), ((16, 16, 16, 16), (2, 4, 4, 4), 2, 5)])
+def test_transfers_with_shared_aggregates(prec, tol, dims, block, n_vec, nrhs):
+    """P^H and P with several CTAs per aggregate (few aggregates, fewer vectors than CTAs) and with one, odd and
+    even batches, against the oracle at the stated bounds."""
+    from oracle.aggregation import Aggregation
+    from oracle.dirac import DiracOperator
+    from paper_1303_1377_gb300 import ddamg
+
+    s, U = _solver(dims, n_vec=n_vec, block=block, precision=getattr(ddamg, "PREC_" + prec))
+    v = synth.random_test_vectors(dims, n_vec, seed=81)
+    x = synth.gaussian_spinors(dims, nrhs, seed=82)
+    agg = Aggregation(DiracOperator(U, dims, -0.4, 1.0).lat, block, v)
+    with s:
+        s.setup_from_vectors(v)
+        e = synth.gaussian_coarse(s.n_coarse, s.coarse_dof, nrhs, seed=83)
+        c, f = s.restrict(x), s.prolong(e)
+    for r in range(nrhs):
+        for got, ref in ((c[r], agg.restrict(x[r])), (f[r], agg.prolong(e[r]))):
+            assert np.max(np.abs(got - ref)) < tol * np.max(np.abs(ref))
