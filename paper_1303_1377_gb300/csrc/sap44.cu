@@ -209,8 +209,261 @@ __global__ void __launch_bounds__(128, 2)
     add_z(0, io, xo, I12());
 }
 
+// ---------------------------------------------------------------------------
+// One right-hand side.  There is no second field to pack, and one CTA of 128 threads per block leaves an SM
+// with one warp per scheduler when there are few blocks; so two threads share a site pair: thread s takes
+// spin s of the projected half spinors in the hops (psi_s and one lower row in, the upper row s and one
+// lower row out) and chirality half s in the site terms, and the two exchange their parts after the hops
+// by shuffles (lanes l and l ^ 16).  One field, one colour, against sap44_kernel with an idle second field: 16^4
+// FP16 operator 45 -> 27 us, FP32 operator 45 -> 31 us; 24^4 151 -> 103 and 159 -> 127 us.
+// ---------------------------------------------------------------------------
+template <int P>
+__device__ __forceinline__ cplx<float> c_fma_ipow(cplx<float> a, cplx<float> b, float g) {  // a + g i^P b
+    const cplx<float> w = ipow<(P & 3)>(b);
+    return mk(fmaf(g, w.re, a.re), fmaf(g, w.im, a.im));
+}
+struct SpinAcc {  // upper row s; lower row s (mu = 2, 3) and lower row 1 - s (mu = 0, 1)
+    cplx<float> up[3], same[3], oth[3];
+};
+// the two threads' factors i^p differ by a sign for mu = 1, 2: sg = +1 for s = 0, -1 for s = 1
+template <int MU, bool FWD, typename PU, typename PL>
+__device__ __forceinline__ void hop_spin(SpinAcc& acc, const PU& up, const PL& low, const cplx<float> (&W)[9], float sg) {
+    using B = SpinB<MU>;
+    constexpr int S = FWD ? 2 : 0;  // h = up -+ i^p low
+    const float f = (MU == 1 || MU == 2) ? sg : 1.f;
+    cplx<float> h[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) h[c] = c_fma_ipow<B::p0 + S>(up(c), low(c), f);
+    cplx<float>(&lo)[3] = MU < 2 ? acc.oth : acc.same;
+    constexpr int HP = (MU < 2 ? B::hp1 : B::hp0) + S;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        cplx<float> g = czero<float>();
+#pragma unroll
+        for (int b = 0; b < 3; ++b) {
+            if (FWD) cmac(g, W[a * 3 + b], h[b]);
+            else cmac_conj(g, W[b * 3 + a], h[b]);
+        }
+        acc.up[a] = acc.up[a] + g;
+        lo[a] = c_fma_ipow<HP>(lo[a], g, f);
+    }
+}
+__device__ __forceinline__ cplx<float> shfl16(cplx<float> a) {
+    return mk(__shfl_xor_sync(0xffffffffu, a.re, 16), __shfl_xor_sync(0xffffffffu, a.im, 16));
+}
+// thread s = 0 gets the upper two spin rows, thread s = 1 the lower two
+__device__ __forceinline__ void spin_exchange(const SpinAcc& acc, int s, cplx<float> (&out)[6]) {
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        const cplx<float> x = shfl16(s ? acc.up[a] : acc.same[a]);  // s = 0 receives row 1, s = 1 a part of row 2
+        const cplx<float> y = shfl16(acc.oth[a]);                   // s = 1 receives a part of row 3
+        out[a] = s ? acc.oth[a] + x : acc.up[a];
+        out[3 + a] = s ? acc.same[a] + y : x;
+    }
+}
+__device__ __forceinline__ void spin_zero(SpinAcc& acc) {
+#pragma unroll
+    for (int k = 0; k < 3; ++k) acc.up[k] = acc.same[k] = acc.oth[k] = czero<float>();
+}
+// y = (block s of the site term) x
+template <typename CF>
+__device__ __forceinline__ void herm6_apply(const CF& cf, const cplx<float> (&x)[6], cplx<float> (&y)[6]) {
+#pragma unroll
+    for (int a = 0; a < 6; ++a) y[a] = cf(a) * x[a];
+    int m = 0;
+#pragma unroll
+    for (int a = 0; a < 6; ++a)
+#pragma unroll
+        for (int b = a + 1; b < 6; ++b) {
+            const cplx<float> e = mk(cf(6 + 2 * m), cf(7 + 2 * m));
+            cmac(y[a], e, x[b]);
+            cmac_conj(y[b], e, x[a]);
+            ++m;
+        }
+}
+__device__ __forceinline__ void herm44_one(const CloverB& cl, int c, int l, int s, const cplx<float> (&x)[6], cplx<float> (&y)[6]) {
+    const float4* q = cl.p + (size_t)c * (18 * 256) + s * (9 * 256) + l;
+    float w[36];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) {
+        const float4 v = __ldg(q + k * 256);
+        w[4 * k] = v.x, w[4 * k + 1] = v.y, w[4 * k + 2] = v.z, w[4 * k + 3] = v.w;
+    }
+    herm6_apply([&](int j) { return w[j]; }, x, y);
+}
+__device__ __forceinline__ void herm44_one(const CloverB16& cl, int c, int l, int s, const cplx<float> (&x)[6], cplx<float> (&y)[6]) {
+    const uint4* q = cl.p + (size_t)c * (10 * 256) + s * (5 * 256) + l;
+    unsigned w[20];
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        const uint4 v = __ldg(q + k * 256);
+        w[4 * k] = v.x, w[4 * k + 1] = v.y, w[4 * k + 2] = v.z, w[4 * k + 3] = v.w;
+    }
+    herm6_apply(
+        [&](int j) {
+            const float2 f = h2f(w[j / 2]);
+            return (j & 1) ? f.y : f.x;
+        },
+        x, y);
+}
+// in-block hops (as hop_pair44: a neighbour outside the block is replaced, with a zero link)
+template <int MU, typename UT>
+__device__ __forceinline__ void hop_pair_one(const UT& U, const cplx<float>* sm, int L, int nb0, int c, int l, int s, float sg, SpinAcc& acc) {
+    constexpr int SH = 2 * (3 - MU), S = 1 << SH;
+    const int y = (L >> SH) & 3;
+    const bool f = y < 3, b = y > 0;
+    const int nf = (f ? L + S : L - S) >> 1, nb = (b ? L - S : L + S) >> 1;
+    const cplx<float>*up = sm + s * (3 * 128), *low = sm + (6 + 3 * (MU < 2 ? 1 - s : s)) * 128;
+    cplx<float> Wf[9], Wb[9];
+    load_link44(Wf, U, c, MU, l, f);
+    load_link44(Wb, U, c, MU, nb0 + nb, b);
+    hop_spin<MU, true>(acc, [&](int k) { return up[k * 128 + nf]; }, [&](int k) { return low[k * 128 + nf]; }, Wf, sg);
+    hop_spin<MU, false>(acc, [&](int k) { return up[k * 128 + nb]; }, [&](int k) { return low[k * 128 + nb]; }, Wb, sg);
+}
+template <typename UT>
+__device__ __forceinline__ void hops_one(const UT& U, const cplx<float>* sm, int L, int nb0, int c, int l, int s, float sg, cplx<float> (&out)[6]) {
+    SpinAcc acc;
+    spin_zero(acc);
+    hop_pair_one<0>(U, sm, L, nb0, c, l, s, sg, acc);
+    hop_pair_one<1>(U, sm, L, nb0, c, l, s, sg, acc);
+    hop_pair_one<2>(U, sm, L, nb0, c, l, s, sg, acc);
+    hop_pair_one<3>(U, sm, L, nb0, c, l, s, sg, acc);
+    spin_exchange(acc, s, out);
+}
+template <int MU, typename UT>
+__device__ __forceinline__ void hop_pair_one_global(const UT& U, const cplx<float>* z, size_t V, int L, int p, int c, int bf, int bb, int s, float sg,
+                                                    SpinAcc& acc) {
+    const cplx<float>*up = z + (size_t)(3 * s) * V, *low = z + (size_t)(6 + 3 * (MU < 2 ? 1 - s : s)) * V;
+    const int f = nbr44<MU, true>(L, p, c, bf), b = nbr44<MU, false>(L, p, c, bb);
+    cplx<float> Wf[9], Wb[9];
+    load_link44(Wf, U, c, MU, (p << 7) | (L >> 1));
+    load_link44(Wb, U, b >> 8, MU, b & 255);
+    hop_spin<MU, true>(acc, [&](int k) { return up[k * V + f]; }, [&](int k) { return low[k * V + f]; }, Wf, sg);
+    hop_spin<MU, false>(acc, [&](int k) { return up[k * V + b]; }, [&](int k) { return low[k * V + b]; }, Wb, sg);
+}
+
+template <typename OpT>
+__global__ void __launch_bounds__(256, 2)
+    sap44_one_kernel(Geom g, OpT op, const cplx<float>* __restrict__ b, cplx<float>* z, int colour, int mr_steps) {
+    constexpr int H = 128;
+    __shared__ cplx<float> SE[12 * H], SO[12 * H];  // even work vector; r_o, then rho, then x_o
+    __shared__ float red[8][3];
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = w * 16 + (lane & 15), s = lane >> 4;
+    const float sg = s ? -1.f : 1.f;
+    const size_t V = g.V, k0 = 6 * s;  // this thread's components 6 s .. 6 s + 5 of its two sites
+    const int c = colour * (g.NB / 2) + blockIdx.x, ie = c * 256 + t, io = ie + H;
+    cplx<float>*me = SE + k0 * H + t, *mo = SO + k0 * H + t;
+    auto add_z = [&](int i, const cplx<float> (&d)[6]) {  // all loads before the first store, as in sap44_kernel
+        cplx<float> u[6];
+#pragma unroll
+        for (int a = 0; a < 6; ++a) u[a] = z[(k0 + a) * V + i];
+#pragma unroll
+        for (int a = 0; a < 6; ++a) z[(k0 + a) * V + i] = u[a] + d[a];
+    };
+    // residual r = b - D z; even sites: SE = A_ee^{-1} r_e, odd sites: SO = r_o
+#pragma unroll 1
+    for (int p = 0; p < 2; ++p) {
+        const int l = p * H + t, i = c * 256 + l, L = lex44_of_local(l);
+        int bn[8];
+#pragma unroll
+        for (int d = 0; d < 8; ++d) bn[d] = __ldg(g.bnbr + d * g.NB + c);
+        SpinAcc acc;
+        spin_zero(acc);
+        hop_pair_one_global<0>(op.U, z, V, L, p, c, bn[0], bn[1], s, sg, acc);
+        hop_pair_one_global<1>(op.U, z, V, L, p, c, bn[2], bn[3], s, sg, acc);
+        hop_pair_one_global<2>(op.U, z, V, L, p, c, bn[4], bn[5], s, sg, acc);
+        hop_pair_one_global<3>(op.U, z, V, L, p, c, bn[6], bn[7], s, sg, acc);
+        cplx<float> hs[6], x[6], y[6];
+        spin_exchange(acc, s, hs);
+#pragma unroll
+        for (int a = 0; a < 6; ++a) x[a] = z[(k0 + a) * V + i];
+        herm44_one(op.clov, c, l, s, x, y);
+#pragma unroll
+        for (int a = 0; a < 6; ++a) x[a] = b[(k0 + a) * V + i] - (y[a] - 0.5f * hs[a]);
+        if (p == 0) {
+            herm44_one(op.clovinv, c, l, s, x, y);
+#pragma unroll
+            for (int a = 0; a < 6; ++a) me[a * H] = y[a];
+        } else {
+#pragma unroll
+            for (int a = 0; a < 6; ++a) mo[a * H] = x[a];
+        }
+    }
+    __syncthreads();  // every read of z in this block is done: z may be updated from here on
+    cplx<float> xo[6];
+#pragma unroll
+    for (int a = 0; a < 6; ++a) xo[a] = me[a * H];
+    add_z(ie, xo);  // the part A_ee^{-1} r_e of x_e, which does not depend on x_o
+#pragma unroll
+    for (int a = 0; a < 6; ++a) xo[a] = czero<float>();
+    const int Le = lex44_of_local(t), Lo = lex44_of_local(H + t);
+    // the passes of sap44_kernel
+#pragma unroll 1
+    for (int it = 0; it <= mr_steps; ++it) {
+        const bool last = it == mr_steps;
+        {
+            cplx<float> sr[6];
+            hops_one(op.U, SE, Lo, 0, c, H + t, s, sg, sr);
+            if (it == 0) {
+#pragma unroll
+                for (int a = 0; a < 6; ++a) mo[a * H] = mo[a * H] + 0.5f * sr[a];
+            } else {
+                cplx<float> rho[6], y[6];
+                float nr = 0.f, ni = 0.f, dd = 0.f;
+#pragma unroll
+                for (int a = 0; a < 6; ++a) rho[a] = mo[a * H];
+                herm44_one(op.clov, c, H + t, s, rho, y);
+#pragma unroll
+                for (int a = 0; a < 6; ++a) {
+                    const cplx<float> v = y[a] + 0.5f * sr[a];
+                    sr[a] = v;
+                    nr += v.re * rho[a].re + v.im * rho[a].im;
+                    ni += v.re * rho[a].im - v.im * rho[a].re;
+                    dd += norm2(v);
+                }
+                nr = warp_sum(nr), ni = warp_sum(ni), dd = warp_sum(dd);
+                if (lane == 0) red[w][0] = nr, red[w][1] = ni, red[w][2] = dd;
+                __syncthreads();
+                nr = ni = dd = 0.f;
+#pragma unroll
+                for (int q = 0; q < 8; ++q) nr += red[q][0], ni += red[q][1], dd += red[q][2];
+                const cplx<float> alpha = dd > tiny_normal<float>() ? mk(nr / dd, ni / dd) : czero<float>();
+#pragma unroll
+                for (int a = 0; a < 6; ++a) {  // x_o += alpha rho, rho -= alpha S rho
+                    cmac(xo[a], alpha, rho[a]);
+                    if (!last) mo[a * H] = rho[a] - alpha * sr[a];
+                }
+            }
+            if (last) {
+#pragma unroll
+                for (int a = 0; a < 6; ++a) mo[a * H] = xo[a];
+            }
+        }
+        __syncthreads();
+        {
+            cplx<float> x[6], y[6];
+            hops_one(op.U, SO, Le, H, c, t, s, sg, x);
+#pragma unroll
+            for (int a = 0; a < 6; ++a) x[a] = (last ? 0.5f : -0.5f) * x[a];
+            herm44_one(op.clovinv, c, t, s, x, y);
+            if (last) add_z(ie, y);
+            else {
+#pragma unroll
+                for (int a = 0; a < 6; ++a) me[a * H] = y[a];
+            }
+        }
+        __syncthreads();
+    }
+    add_z(io, xo);
+}
+
 template <typename OpT>
 int launch_sap44(const Geom& g, const OpT& op, const cplx<float>* b, cplx<float>* z, int colour, int nrhs, int mr_steps, cudaStream_t st) {
+    if (nrhs == 1) {
+        sap44_one_kernel<OpT><<<(unsigned)(g.NB / 2), 256, 0, st>>>(g, op, b, z, colour, mr_steps);
+        DD_CHECK_LAUNCH();
+        return 0;
+    }
     const size_t smem = 24 * 128 * sizeof(float4) + 12 * sizeof(float2);
     // set once per kernel instance (a function-local static initialiser is thread safe)
     static const bool attr = [] {
