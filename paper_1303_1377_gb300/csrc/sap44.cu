@@ -10,7 +10,7 @@
 // What bounds it: the packed multiply-adds (two cycles each) hold the FMA pipe about 60% busy in the MR
 // steps; the residual at the start waits on its neighbours' spinors.  12 fields on 24^4, one colour,
 // FP16 operator: 740 us (29 TFLOP/s) against 1347 us for one right-hand side per thread, four per CTA
-// (512 threads, 128 registers); FP32 operator 740 against 1399 us; one field 151 against 212 us.  Tried
+// (512 threads, 128 registers); FP32 operator 740 against 1399 us.  Few blocks, or one field: sap44_one_kernel below.  Tried
 // and slower (same case): four right-hand sides per CTA 778 us, six 806 us; x_o in shared memory
 // (+12%); the links in shared memory as FP32 (+5%); two threads per site split by spin 781 us; own z
 // and the faces staged through shared memory (+15%).
@@ -210,8 +210,8 @@ __global__ void __launch_bounds__(128, 2)
 }
 
 // ---------------------------------------------------------------------------
-// One right-hand side.  There is no second field to pack, and one CTA of 128 threads per block leaves an SM
-// with one warp per scheduler when there are few blocks; so two threads share a site pair: thread s takes
+// One right-hand side per CTA (grid.y = right-hand sides): one field has no second one to pack, and with few
+// blocks a CTA of 128 threads leaves an SM one warp per scheduler; so two threads share a site pair: thread s takes
 // spin s of the projected half spinors in the hops (psi_s and one lower row in, the upper row s and one
 // lower row out) and chirality half s in the site terms, and the two exchange their parts after the hops
 // by shuffles (lanes l and l ^ 16).  One field, one colour, against sap44_kernel with an idle second field: 16^4
@@ -344,13 +344,15 @@ __device__ __forceinline__ void hop_pair_one_global(const UT& U, const cplx<floa
 
 template <typename OpT>
 __global__ void __launch_bounds__(256, 2)
-    sap44_one_kernel(Geom g, OpT op, const cplx<float>* __restrict__ b, cplx<float>* z, int colour, int mr_steps) {
+    sap44_one_kernel(Geom g, OpT op, const cplx<float>* __restrict__ bsrc, cplx<float>* zsrc, int colour, int mr_steps) {
     constexpr int H = 128;
     __shared__ cplx<float> SE[12 * H], SO[12 * H];  // even work vector; r_o, then rho, then x_o
     __shared__ float red[8][3];
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, t = w * 16 + (lane & 15), s = lane >> 4;
     const float sg = s ? -1.f : 1.f;
     const size_t V = g.V, k0 = 6 * s;  // this thread's components 6 s .. 6 s + 5 of its two sites
+    const cplx<float>* b = bsrc + (size_t)blockIdx.y * 12 * V;
+    cplx<float>* z = zsrc + (size_t)blockIdx.y * 12 * V;
     const int c = colour * (g.NB / 2) + blockIdx.x, ie = c * 256 + t, io = ie + H;
     cplx<float>*me = SE + k0 * H + t, *mo = SO + k0 * H + t;
     auto add_z = [&](int i, const cplx<float> (&d)[6]) {  // all loads before the first store, as in sap44_kernel
@@ -459,8 +461,13 @@ __global__ void __launch_bounds__(256, 2)
 
 template <typename OpT>
 int launch_sap44(const Geom& g, const OpT& op, const cplx<float>* b, cplx<float>* z, int colour, int nrhs, int mr_steps, cudaStream_t st) {
-    if (nrhs == 1) {
-        sap44_one_kernel<OpT><<<(unsigned)(g.NB / 2), 256, 0, st>>>(g, op, b, z, colour, mr_steps);
+    // Few blocks: one CTA per block and field while they all fit on the chip, one per SM (FP32 operator) or two (FP16,
+    // half the L1 footprint).  us per colour, one field per CTA / pairs: 8^4 (8 blocks) 12 fields 27 / 39 (FP16), 31 / 41
+    // (FP32); 16x8^3 12 fields (192 CTAs) 41 / 45, 45 / 44; 16^4 two fields (256 CTAs) 42 / 48, 47 / 48; three 61 / 62,
+    // 72 / 63; 24^4 two 177 / 159.
+    const long long slots = std::is_same<OpT, FineOpB16>::value ? 2 * 152 : 152;
+    if (nrhs == 1 || (long long)(g.NB / 2) * nrhs <= slots) {
+        sap44_one_kernel<OpT><<<dim3((unsigned)(g.NB / 2), (unsigned)nrhs), 256, 0, st>>>(g, op, b, z, colour, mr_steps);
         DD_CHECK_LAUNCH();
         return 0;
     }

@@ -165,6 +165,26 @@ def test_half_restriction_of_fields_of_very_different_size(dims, n_vec, nrhs):
         assert np.max(np.abs(got[r] - ref)) <= 4e-3 * np.max(np.abs(ref))
 
 
+@pytest.mark.parametrize("prec,tol", [("single", 1e-6), ("half", 2e-3)])
+@pytest.mark.parametrize("nrhs", [2, 3])
+def test_sap_on_both_sides_of_the_line_between_its_kernels(prec, tol, nrhs):
+    """16^4 has 128 blocks per colour: two and three fields lie on either side of the line between one field per
+    CTA and pairs of fields.  The first and the last field against the oracle, at the stated bounds."""
+    from oracle.dirac import DiracOperator
+    from oracle.sap import SAP
+    from paper_1303_1377_gb300 import ddamg
+
+    dims = (16, 16, 16, 16)
+    s, U = _solver(dims, n_vec=4, precision={"single": ddamg.PREC_SINGLE, "half": ddamg.PREC_HALF}[prec], mr_steps=2)
+    with s:
+        b = synth.gaussian_spinors(dims, nrhs, seed=25)
+        got = s.apply_sap(b, 1)
+    sap = SAP(DiracOperator(U, dims, -0.4, 1.0), (4, 4, 4, 4), mr_steps=2)
+    for r in (0, nrhs - 1):
+        ref = sap.apply(b[r], 1)
+        assert np.max(np.abs(got[r] - ref)) < tol * np.max(np.abs(ref))
+
+
 @pytest.mark.parametrize("prec,tol", [("DOUBLE", 1e-13), ("SINGLE", 1e-6)])
 @pytest.mark.parametrize("dims,block,n_vec,nrhs", [((4, 4, 4, 4), (2, 2, 2, 2), 1, 1), ((8, 8, 8, 8), (4, 4, 4, 4), 3, 3),
                                                    ((16, 8, 8, 8), (2, 2, 4, 4), 7, 1), ((16, 16, 16, 16), (2, 4, 4, 4), 2, 5)])
