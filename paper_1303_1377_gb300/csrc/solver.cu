@@ -2146,6 +2146,18 @@ static int prolong_T(ddamg_handle* h, const double* in, double* out, int n_rhs) 
     cplx<T>* a = h->ws_fine[4].as<cplx<T>>();
     cplx<T>* o = a + cn * n_rhs;
     DD_TRY(coarse_in<T>(h, in, n_rhs, a));
+    if constexpr (std::is_same<T, float>::value) {
+        if (h->half() && prolong_tc_lex_supported(h->g, h->N)) {  // the kernel writes the caller's layout itself
+            void* dv;
+            bool host;
+            DD_TRY(stage_out_ptr(h->ws_io[1], out, sizeof(cplx<double>) * fld * n_rhs, &dv, &host));
+            {
+                Prof pr(h, PF_PROLONG, (double)h->V * (12.0 * h->N * 4 + 12.0 * n_rhs * 16));
+                DD_TRY(launch_prolong_tc_lex(h->g, h->P16, h->N, a, reinterpret_cast<cplx<double>*>(dv), h->d_lex_of, n_rhs, h->stream));
+            }
+            return finish_out(h, out, dv, sizeof(cplx<double>) * fld * n_rhs, host);
+        }
+    }
     DD_TRY(prolong_<T>(h, a, o, n_rhs));
     return fine_out<T>(h, o, out, n_rhs);
 }

@@ -206,3 +206,28 @@ def test_transfers_with_shared_aggregates(prec, tol, dims, block, n_vec, nrhs):
     for r in range(nrhs):
         for got, ref in ((c[r], agg.restrict(x[r])), (f[r], agg.prolong(e[r]))):
             assert np.max(np.abs(got - ref)) < tol * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dims,block,n_vec,nrhs", [((4, 4, 4, 4), (2, 2, 2, 2), 4, 3), ((8, 4, 4, 12), (4, 2, 2, 2), 8, 1),
+                                                   ((8, 8, 16, 8), (4, 4, 4, 4), 20, 17)])
+def test_half_prolongation_by_block_and_right_hand_sides(dims, block, n_vec, nrhs):
+    """P on half-precision handles: blocks of 16 sites (result through the internal layout), of 32 and of 256 sites
+    (written in the caller's layout), one field and a second launch of five, fields from 1e-30 to 1e30, each to the
+    stated 4e-3 of its own result's maximum."""
+    from oracle.aggregation import Aggregation
+    from oracle.dirac import DiracOperator
+    from paper_1303_1377_gb300 import ddamg
+
+    s, U = _solver(dims, block=block, n_vec=n_vec, precision=ddamg.PREC_HALF)
+    v = synth.random_test_vectors(dims, n_vec, seed=73)
+    agg = Aggregation(DiracOperator(U, dims, -0.4, 1.0).lat, block, v)
+    rng = np.random.default_rng(74)
+    nb = int(np.prod(dims)) // int(np.prod(block))
+    e = rng.standard_normal((nrhs, nb, 2 * n_vec)) + 1j * rng.standard_normal((nrhs, nb, 2 * n_vec))
+    e *= 10.0 ** np.linspace(-30, 30, nrhs)[:, None, None]
+    with s:
+        s.setup_from_vectors(v)
+        got = s.prolong(e)
+    for r in range(nrhs):
+        ref = agg.prolong(e[r])
+        assert np.max(np.abs(np.reshape(got[r], ref.shape) - ref)) <= 4e-3 * np.max(np.abs(ref))
