@@ -1,33 +1,34 @@
 // FP32 Dslash on 4^4 blocks for two or more right-hand sides.
 //
-// Bound by the latency of the neighbours' spinors: three quarters of the time of 12 fields on 32^4 is spent
-// waiting for them (12 warps per SM at 168 registers).  Against one right-hand side per thread on the
-// [component][site] operator (24 warps, 80 registers) the loads in flight are the same and the
-// instructions per field 0.55x: 12 fields of 32^4 1646 -> 1290 us (2.3 TB/s of operator and fields read and
-// written once).  Three CTAs per SM (96 registers) spill: 1900 us.
-#include <algorithm>
+// Bound by the latency of the neighbours' spinors.  A CTA of 128 threads covers half a block (64 sites of
+// either parity) and one pair of right-hand sides: 128 registers leave 16 warps on an SM, and most in-block
+// neighbours are sites of the same CTA, so their spinors hit L1.  12 fields of 32^4, the call: 1785 us; a CTA of
+// 32 sites and up to six pairs (168 registers, 12 warps, operator shared through L1) 1980 us, whole blocks
+// (256 threads) 1806 us, quarter blocks 1870 us; 226 registers, two CTAs per SM, 1972 us; 12 fields of 24^4
+// 600 against 648 us, two of 16^3 x 32 92 against 90 us.  One right-hand side per thread (24 warps, 80
+// registers) took 1646 us for the kernel alone against 1290 us in the six-pair form.
 #include <type_traits>
 
 #include "ops44.cuh"
 
 namespace ddamg {
 
-// out = D in (RESID: out = b - D in).  Thread (x, y): site x of 32 sites of one block, right-hand sides
-// 2 y and 2 y + 1 of the CTA's, in packed FP32 instructions; the warps of a CTA share the links and site
-// terms of their sites through L1.  The CTAs walk the blocks in lexicographic order, red and black
+// out = D in (RESID: out = b - D in).  One thread per site, two right-hand sides in packed FP32
+// instructions.  The pairs of right-hand sides of a half block follow one another, so the links and site
+// terms come from L2 after the first; the CTAs walk the blocks in lexicographic order, red and black
 // interleaved, so that a block and its neighbours in three of the four directions are read close
 // together in time and the neighbours' spinors are still in L2.
 // lex != null: out is in the caller's layout ([field][site lex[i]][12], 16-byte aligned): a site's
 // components leave as whole 16-byte words, and no separate pass has to reorder the field.
 template <bool RESID>
-__global__ void __launch_bounds__(192, 2)
+__global__ void __launch_bounds__(128, 4)
     dslash44_pair_kernel(Geom g, FineOpB op, const cplx<float>* __restrict__ in, const cplx<float>* __restrict__ b, cplx<float>* __restrict__ out,
                          const int* __restrict__ lex, int nrhs) {
-    const int r0 = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
-    if (r0 >= nrhs) return;
+    const unsigned pairs = (unsigned)(nrhs + 1) / 2, sub = blockIdx.x / pairs;
+    const int r0 = 2 * (int)(blockIdx.x % pairs);
     const bool two = r0 + 1 < nrhs;  // an odd batch computes its last right-hand side twice and stores it once
-    const int c = __ldg(g.blex + (blockIdx.x >> 3));
-    const int l = (blockIdx.x & 7) * 32 + threadIdx.x, i = c * 256 + l, V = g.V;
+    const int c = __ldg(g.blex + (sub >> 1));
+    const int l = (threadIdx.x >> 6) * 128 + (sub & 1) * 64 + (threadIdx.x & 63), i = c * 256 + l, V = g.V;
     const int L = lex44_of_local(l), p = l >> 7;
     int bn[8];
 #pragma unroll
@@ -76,8 +77,7 @@ __global__ void __launch_bounds__(192, 2)
 
 int launch_dslash44_pair(const Geom& g, const FineOpB& op, const cplx<float>* in, const cplx<float>* b, cplx<float>* out, const int* lex,
                          int nrhs, cudaStream_t st) {
-    const int pairs = (nrhs + 1) / 2, ry = std::min(pairs, 6);
-    const dim3 grid((unsigned)g.NB * 8, (unsigned)ceil_div(pairs, ry)), block(32, ry);
+    const unsigned grid = 2u * (unsigned)g.NB * (unsigned)((nrhs + 1) / 2), block = 128;
     if (b)
         dslash44_pair_kernel<true><<<grid, block, 0, st>>>(g, op, in, b, out, lex, nrhs);
     else
