@@ -31,8 +31,9 @@ __device__ __forceinline__ void hop_pair_nb(const UT& U, const cplx<Ts>* __restr
     hop_acc<MU, false>(acc, pn, W);
 }
 
-// out = D in (RESID: out = b - D in) on 4^4 blocks.  CTA = 32 sites of one block x ry right-hand
-// sides (one warp per right-hand side, sharing the links and site terms through L1).  The CTAs walk
+// out = D in (RESID: out = b - D in) on 4^4 blocks, FP64 and single FP32 fields (two and more FP32
+// fields: dslash44.cu).  CTA = 32 sites of one block x ry right-hand sides (one warp per right-hand
+// side, sharing the links and site terms through L1).  The CTAs walk
 // the blocks in lexicographic block order, red and black interleaved, so that a block and its
 // neighbours in three of the four directions are read close together in time and the neighbours'
 // spinors are still in L2.

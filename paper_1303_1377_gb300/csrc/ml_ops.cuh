@@ -439,16 +439,16 @@ struct MLHostExec {
 };
 
 // one SAP colour step of ml_sap as a single kernel (ml_sap.cu): FP32, blocks with as many even as
-// odd sites, at most 384 (block-half sites x components) threads and the six half-block MR vectors
-// of 12 right-hand sides within shared memory
+// odd sites, at most 341 pairs (block-half site, component) (three threads each in a CTA) and the six
+// half-block MR vectors of 12 right-hand sides within shared memory
+bool ml_sap_fused_supported(const MLView<float>& v);
+int launch_ml_sap_fused(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps,
+                        cudaStream_t st);
 // the same step on tensor cores for the FP16 copies in fragment order (ml_sap_tc.cu), and their packing
 // from nblk FP64 column-major nc x nc blocks
 bool ml_sap_tc_supported(int nc, int Vb1, int Vb1e);
 int launch_ml_sap_tc(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps, cudaStream_t st);
 int pack_ml_frag(const double* in, void* out, size_t nblk, int nc, cudaStream_t st);
-bool ml_sap_fused_supported(const MLView<float>& v);
-int launch_ml_sap_fused(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps,
-                        cudaStream_t st);
 
 // ---------------------------------------------------------------------------
 // orchestration
