@@ -162,12 +162,18 @@ __global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __
 // Two right-hand sides per thread in packed FP32 (f32x2.cuh): the same double-word operations, each issued
 // once for two fields, with the links' and site terms' words loaded once for two.
 //
-// Bound by the latency of its chains at eight warps per SM (254 registers; FMA pipe 42% busy): a
-// double-word multiply-add is 12 packed instructions of two cycles.  The loop over the eight directions is
-// rolled (one hop is about 20 KB of code) with the spin structure as run-time selects and sign flips on the
-// integer pipe; accumulators stay in registers.  FP64 instructions issue at 1/64 of the FP32 rate,
+// Two threads share a site: thread s takes row s of the projected half spinors in the hops (the upper row s and
+// one lower row out) and chirality half s of the site term; their parts meet by shuffles after the last hop.
+// Bound by the latency of its chains (a double-word multiply-add is 12 packed instructions of two cycles) at 12
+// warps per SM (168 registers); one thread per site held 24 accumulators and ran 8 warps of 254 registers: 12
+// fields of 24^4, the call, 3600 -> 3280 us, five of 8x16x8x24 184 -> 168 us, two of
+// 16^3 x 32 271 -> 278 us; error against 64 bits 5.8e-15 both.
+// The accumulators parked in shared memory during the site term: 3410 us; four CTAs per SM (spills): 3530 us; the
+// site term added straight onto -acc / 2: 2910 us, but the error rises to 7.5e-15.
+// The loop over the eight directions is rolled (one hop is about 10 KB of code) with the spin structure as
+// run-time selects and sign flips on the integer pipe.  FP64 instructions issue at 1/64 of the FP32 rate,
 // conversions included: y - acc / 2 is summed in FP32 words and takes one FP64 addition a number (formed in
-// FP64 from its four words the call took 0.94 ms longer).  12 fields of 24^4: 3703 -> 3220 us.
+// FP64 from its four words the call took 0.94 ms longer).
 // ---------------------------------------------------------------------------
 namespace {
 
@@ -226,125 +232,132 @@ __device__ __forceinline__ unsigned sign_im(int p) { return (p & 2) ? 0x80000000
 }  // namespace
 
 template <bool OUT_DW>
-__global__ void __launch_bounds__(128, 2) dslash_dw_pair_kernel(Geom g, const float4* __restrict__ U, const float2* __restrict__ clov,
+__global__ void __launch_bounds__(128, 3) dslash_dw_pair_kernel(Geom g, const float4* __restrict__ U, const float2* __restrict__ clov,
                                                                 const cplx<float>* __restrict__ in, void* __restrict__ outp, int nrhs) {
     const int r0 = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
-    const int i = blockIdx.x * 32 + threadIdx.x;
-    if (i >= g.V || r0 >= nrhs) return;
+    const int lane = threadIdx.x, s = lane >> 4, i = blockIdx.x * 16 + (lane & 15);  // V is a multiple of 16
+    if (r0 >= nrhs) return;  // (a whole warp)
     const bool two = r0 + 1 < nrhs;  // an odd batch computes its last right-hand side twice and stores it once
     const size_t V = g.V, o0 = (size_t)r0 * 12 * V, o1 = o0 + (two ? 12 * V : 0);
     const cplx<float>*z0 = in + o0, *z1 = in + o1;
-    cdw2 acc[12];
+    cdw2 up[3], same[3], oth[3];
 #pragma unroll
-    for (int k = 0; k < 12; ++k) acc[k] = cdw2_zero();
+    for (int k = 0; k < 3; ++k) up[k] = same[k] = oth[k] = cdw2_zero();
 #pragma unroll 1
     for (int d = 0; d < 8; ++d) {
         const int nb = fine_nbr(g, i, d), mu = d >> 1;
         const bool fwd = (d & 1) == 0;
         const unsigned sf = fwd ? 0x80000000u : 0u;  // h = up -+ i^p low
-        const bool c0 = c_spinb[mu][0], c1 = c_spinb[mu][2], hc0 = c_spinb[mu][4], hc1 = c_spinb[mu][6];
-        const int p0 = c_spinb[mu][1], p1 = c_spinb[mu][3], hp0 = c_spinb[mu][5], hp1 = c_spinb[mu][7];
-        cdw2 h[2][3];
+        // row s of B_mu reads lower row c with factor i^p; the same lower row takes i^hp of the product
+        const int c = c_spinb[mu][2 * s], p = c_spinb[mu][2 * s + 1];
+        const int hp = c_spinb[mu][5 + 2 * c];  // (lower row c: B_mu and B_mu^H both keep the spins or both swap them)
+        const size_t ro = (size_t)(3 * s) * V + nb, rl = (size_t)(6 + 3 * c) * V + nb;
+        const unsigned mr = sign_re(p) ^ sf, mi = sign_im(p) ^ sf;
+        cdw2 h[3];
 #pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const c2 u0 = c2pair(z0[c * V + nb], z1[c * V + nb]), u1 = c2pair(z0[(3 + c) * V + nb], z1[(3 + c) * V + nb]);
-            const c2 l2 = c2pair(z0[(6 + c) * V + nb], z1[(6 + c) * V + nb]), l3 = c2pair(z0[(9 + c) * V + nb], z1[(9 + c) * V + nb]);
-            const c2 b0 = {sel2(c0, l3.re, l2.re), sel2(c0, l3.im, l2.im)}, b1 = {sel2(c1, l3.re, l2.re), sel2(c1, l3.im, l2.im)};
-            h[0][c].re = two_sum2(u0.re, flip2(sel2(p0 & 1, b0.im, b0.re), sign_re(p0) ^ sf));
-            h[0][c].im = two_sum2(u0.im, flip2(sel2(p0 & 1, b0.re, b0.im), sign_im(p0) ^ sf));
-            h[1][c].re = two_sum2(u1.re, flip2(sel2(p1 & 1, b1.im, b1.re), sign_re(p1) ^ sf));
-            h[1][c].im = two_sum2(u1.im, flip2(sel2(p1 & 1, b1.re, b1.im), sign_im(p1) ^ sf));
+        for (int k = 0; k < 3; ++k) {
+            const c2 u = c2pair(z0[ro + k * V], z1[ro + k * V]), l = c2pair(z0[rl + k * V], z1[rl + k * V]);
+            h[k].re = two_sum2(u.re, flip2(sel2(p & 1, l.im, l.re), mr));
+            h[k].im = two_sum2(u.im, flip2(sel2(p & 1, l.re, l.im), mi));
         }
         const float4* W = U + (size_t)(mu * 9) * V + (fwd ? i : nb);
         const unsigned cj = fwd ? 0u : 0x80000000u;  // W^H backwards
         const size_t sa = (fwd ? 3 : 1) * V, sb = (fwd ? 1 : 3) * V;
+        const unsigned gr = sign_re(hp) ^ sf, gi = sign_im(hp) ^ sf;
+        const bool swap = mu < 2;
 #pragma unroll
         for (int a = 0; a < 3; ++a) {
-            cdw2 t[2];
-            t[0] = t[1] = cdw2_zero();
+            cdw2 t = cdw2_zero();
 #pragma unroll
             for (int b = 0; b < 3; ++b) {
                 const float4 w = __ldg(W + a * sa + b * sb);
                 const float ih = flip(w.z, cj), il = flip(w.w, cj);
                 const float2 rh = f2dup(w.x), nrh = f2dup(-w.x), nrl = f2dup(-w.y);
                 const float2 ph = f2dup(ih), nh = f2dup(-ih), pl = f2dup(il), nl = f2dup(-il);
-#pragma unroll
-                for (int s = 0; s < 2; ++s) {
-                    dw2_mac(t[s].re, rh, nrh, nrl, h[s][b].re);
-                    dw2_mac(t[s].re, nh, ph, pl, h[s][b].im);
-                    dw2_mac(t[s].im, rh, nrh, nrl, h[s][b].im);
-                    dw2_mac(t[s].im, ph, nh, nl, h[s][b].re);
-                }
+                dw2_mac(t.re, rh, nrh, nrl, h[b].re);
+                dw2_mac(t.re, nh, ph, pl, h[b].im);
+                dw2_mac(t.im, rh, nrh, nrl, h[b].im);
+                dw2_mac(t.im, ph, nh, nl, h[b].re);
             }
-#pragma unroll
-            for (int s = 0; s < 2; ++s) {
-                t[s].re = dw2_norm(t[s].re), t[s].im = dw2_norm(t[s].im);
-                acc[s * 3 + a].re = dw2_add(acc[s * 3 + a].re, t[s].re);
-                acc[s * 3 + a].im = dw2_add(acc[s * 3 + a].im, t[s].im);
-            }
-            const cdw2 x0 = {sel_flip(hc0, t[1].re, t[0].re, 0u), sel_flip(hc0, t[1].im, t[0].im, 0u)};
-            const cdw2 x1 = {sel_flip(hc1, t[1].re, t[0].re, 0u), sel_flip(hc1, t[1].im, t[0].im, 0u)};
-            acc[6 + a].re = dw2_add(acc[6 + a].re, sel_flip(hp0 & 1, x0.im, x0.re, sign_re(hp0) ^ sf));
-            acc[6 + a].im = dw2_add(acc[6 + a].im, sel_flip(hp0 & 1, x0.re, x0.im, sign_im(hp0) ^ sf));
-            acc[9 + a].re = dw2_add(acc[9 + a].re, sel_flip(hp1 & 1, x1.im, x1.re, sign_re(hp1) ^ sf));
-            acc[9 + a].im = dw2_add(acc[9 + a].im, sel_flip(hp1 & 1, x1.re, x1.im, sign_im(hp1) ^ sf));
+            t.re = dw2_norm(t.re), t.im = dw2_norm(t.im);
+            up[a].re = dw2_add(up[a].re, t.re), up[a].im = dw2_add(up[a].im, t.im);
+            const dw2 lr = sel_flip(hp & 1, t.im, t.re, gr), li = sel_flip(hp & 1, t.re, t.im, gi);
+            if (swap) oth[a].re = dw2_add(oth[a].re, lr), oth[a].im = dw2_add(oth[a].im, li);
+            else same[a].re = dw2_add(same[a].re, lr), same[a].im = dw2_add(same[a].im, li);
         }
     }
-    // site term, one chirality half at a time (a packed hermitian 6x6 block of double-word entries)
-#pragma unroll
-    for (int hb = 0; hb < 2; ++hb) {
-        c2 x[6];
-        cdw2 y[6];
-        const float2* base = clov + (size_t)(hb * 36) * V + i;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-            x[a] = c2pair(z0[(hb * 6 + a) * V + i], z1[(hb * 6 + a) * V + i]);
-            const float2 e = __ldg(base + a * V);
-            y[a] = cdw2_zero();
-            dw2_macf(y[a].re, f2dup(e.x), f2dup(-e.x), f2dup(-e.y), x[a].re);
-            dw2_macf(y[a].im, f2dup(e.x), f2dup(-e.x), f2dup(-e.y), x[a].im);
-        }
-        int q = 0;
-#pragma unroll
-        for (int a = 0; a < 6; ++a) {
-#pragma unroll
-            for (int b = a + 1; b < 6; ++b) {
-                const float2 er = __ldg(base + (6 + 2 * q) * V), ei = __ldg(base + (7 + 2 * q) * V);
-                const float2 rh = f2dup(er.x), nrh = f2dup(-er.x), nrl = f2dup(-er.y);
-                const float2 ph = f2dup(ei.x), nh = f2dup(-ei.x), pl = f2dup(ei.y), nl = f2dup(-ei.y);
-                // y[a] += m x[b];  y[b] += conj(m) x[a]
-                dw2_macf(y[a].re, rh, nrh, nrl, x[b].re);
-                dw2_macf(y[a].re, nh, ph, pl, x[b].im);
-                dw2_macf(y[a].im, rh, nrh, nrl, x[b].im);
-                dw2_macf(y[a].im, ph, nh, nl, x[b].re);
-                dw2_macf(y[b].re, rh, nrh, nrl, x[a].re);
-                dw2_macf(y[b].re, ph, nh, nl, x[a].im);
-                dw2_macf(y[b].im, rh, nrh, nrl, x[a].im);
-                dw2_macf(y[b].im, nh, ph, pl, x[a].re);
-                ++q;
-            }
-        }
-        const float2 mh = f2dup(-0.5f);
-        // y - acc / 2: the sum of the high words and its exact error, with the low words added to that error by
-        // error-free sums, so that only the last word is rounded
-        auto sub = [&](const dw2& u, const dw2& v) -> dw2 {
-            const dw2 p = two_sum2(u.h, f2mul(mh, v.h)), q = two_sum2(u.l, f2mul(mh, v.l)), t = two_sum2(p.l, q.h);
-            const float2 m = f2add(t.h, f2add(t.l, q.l)), h = f2add(p.h, m);
-            return {h, f2add(f2sub(m, f2sub(h, p.h)), f2add(f2sub(t.h, m), f2add(t.l, q.l)))};
+    // thread s = 0 takes the upper two spin rows, thread s = 1 the lower two
+    cdw2 acc[6];
+    {
+        auto sh = [](const dw2& v) -> dw2 {
+            return {make_float2(__shfl_xor_sync(0xffffffffu, v.h.x, 16), __shfl_xor_sync(0xffffffffu, v.h.y, 16)),
+                    make_float2(__shfl_xor_sync(0xffffffffu, v.l.x, 16), __shfl_xor_sync(0xffffffffu, v.l.y, 16))};
         };
+        auto pick = [&](const dw2& v, const dw2& w) -> dw2 { return {sel2(s, v.h, w.h), sel2(s, v.l, w.l)}; };
 #pragma unroll
-        for (int a = 0; a < 6; ++a) {
-            const dw2 re = sub(y[a].re, acc[hb * 6 + a].re), im = sub(y[a].im, acc[hb * 6 + a].im);
-            const size_t k = (size_t)(hb * 6 + a) * V + i;
-            if (OUT_DW) {
-                float4* o = reinterpret_cast<float4*>(outp);
-                o[o0 + k] = make_float4(re.h.x, re.l.x, im.h.x, im.l.x);
-                if (two) o[o1 + k] = make_float4(re.h.y, re.l.y, im.h.y, im.l.y);
-            } else {
-                cplx<double>* o = reinterpret_cast<cplx<double>*>(outp);
-                o[o0 + k] = mk((double)re.h.x + (double)re.l.x, (double)im.h.x + (double)im.l.x);
-                if (two) o[o1 + k] = mk((double)re.h.y + (double)re.l.y, (double)im.h.y + (double)im.l.y);
-            }
+        for (int a = 0; a < 3; ++a) {
+            auto part = [&](const dw2& u, const dw2& sa, const dw2& ot, dw2& lo, dw2& hi) {
+                const dw2 x = sh(pick(u, sa)), z = sh(ot);  // for s = 0: x = row 1; for s = 1: parts of rows 2 and 3
+                lo = pick(dw2_add(ot, x), u);
+                hi = pick(dw2_add(sa, z), x);
+            };
+            part(up[a].re, same[a].re, oth[a].re, acc[a].re, acc[3 + a].re);
+            part(up[a].im, same[a].im, oth[a].im, acc[a].im, acc[3 + a].im);
+        }
+    }
+    // the site term of this thread's chirality half (a packed hermitian 6x6 block of double-word entries)
+    c2 x[6];
+    cdw2 y[6];
+    const float2* base = clov + (size_t)(s * 36) * V + i;
+    const size_t k0 = (size_t)(6 * s) * V + i;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+        x[a] = c2pair(z0[k0 + a * V], z1[k0 + a * V]);
+        const float2 e = __ldg(base + a * V);
+        y[a] = cdw2_zero();
+        dw2_macf(y[a].re, f2dup(e.x), f2dup(-e.x), f2dup(-e.y), x[a].re);
+        dw2_macf(y[a].im, f2dup(e.x), f2dup(-e.x), f2dup(-e.y), x[a].im);
+    }
+    int q = 0;
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+#pragma unroll
+        for (int b = a + 1; b < 6; ++b) {
+            const float2 er = __ldg(base + (6 + 2 * q) * V), ei = __ldg(base + (7 + 2 * q) * V);
+            const float2 rh = f2dup(er.x), nrh = f2dup(-er.x), nrl = f2dup(-er.y);
+            const float2 ph = f2dup(ei.x), nh = f2dup(-ei.x), pl = f2dup(ei.y), nl = f2dup(-ei.y);
+            // y[a] += m x[b];  y[b] += conj(m) x[a]
+            dw2_macf(y[a].re, rh, nrh, nrl, x[b].re);
+            dw2_macf(y[a].re, nh, ph, pl, x[b].im);
+            dw2_macf(y[a].im, rh, nrh, nrl, x[b].im);
+            dw2_macf(y[a].im, ph, nh, nl, x[b].re);
+            dw2_macf(y[b].re, rh, nrh, nrl, x[a].re);
+            dw2_macf(y[b].re, ph, nh, nl, x[a].im);
+            dw2_macf(y[b].im, rh, nrh, nrl, x[a].im);
+            dw2_macf(y[b].im, nh, ph, pl, x[a].re);
+            ++q;
+        }
+    }
+    const float2 mh = f2dup(-0.5f);
+    // y - acc / 2: the sum of the high words and its exact error, with the low words added to that error by
+    // error-free sums, so that only the last word is rounded
+    auto sub = [&](const dw2& u, const dw2& v) -> dw2 {
+        const dw2 p = two_sum2(u.h, f2mul(mh, v.h)), q = two_sum2(u.l, f2mul(mh, v.l)), t = two_sum2(p.l, q.h);
+        const float2 m = f2add(t.h, f2add(t.l, q.l)), h = f2add(p.h, m);
+        return {h, f2add(f2sub(m, f2sub(h, p.h)), f2add(f2sub(t.h, m), f2add(t.l, q.l)))};
+    };
+#pragma unroll
+    for (int a = 0; a < 6; ++a) {
+        const dw2 re = sub(y[a].re, acc[a].re), im = sub(y[a].im, acc[a].im);
+        const size_t k = k0 + a * V;
+        if (OUT_DW) {
+            float4* o = reinterpret_cast<float4*>(outp);
+            o[o0 + k] = make_float4(re.h.x, re.l.x, im.h.x, im.l.x);
+            if (two) o[o1 + k] = make_float4(re.h.y, re.l.y, im.h.y, im.l.y);
+        } else {
+            cplx<double>* o = reinterpret_cast<cplx<double>*>(outp);
+            o[o0 + k] = mk((double)re.h.x + (double)re.l.x, (double)im.h.x + (double)im.l.x);
+            if (two) o[o1 + k] = mk((double)re.h.y + (double)re.l.y, (double)im.h.y + (double)im.l.y);
         }
     }
 }
@@ -353,7 +366,7 @@ int launch_dslash_dw(const Geom& g, const float4* U, const float2* clov, const c
                      cudaStream_t st) {
     if (nrhs >= 2) {
         const int pairs = (nrhs + 1) / 2, ry = std::min(pairs, 4);
-        const dim3 grid((unsigned)ceil_div(g.V, 32), (unsigned)ceil_div(pairs, ry)), block(32, ry);
+        const dim3 grid((unsigned)(g.V / 16), (unsigned)ceil_div(pairs, ry)), block(32, ry);
         if (out_dw) dslash_dw_pair_kernel<true><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
         else dslash_dw_pair_kernel<false><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
         DD_CHECK_LAUNCH();
