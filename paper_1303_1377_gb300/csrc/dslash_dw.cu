@@ -166,10 +166,10 @@ __global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __
 // one lower row out) and chirality half s of the site term; their parts meet by shuffles after the last hop.
 // Bound by the latency of its chains (a double-word multiply-add is 12 packed instructions of two cycles) at 12
 // warps per SM (168 registers); one thread per site held 24 accumulators and ran 8 warps of 254 registers: 12
-// fields of 24^4, the call, 3600 -> 3280 us, five of 8x16x8x24 184 -> 168 us, two of
-// 16^3 x 32 271 -> 278 us; error against 64 bits 5.8e-15 both.
-// The accumulators parked in shared memory during the site term: 3410 us; four CTAs per SM (spills): 3530 us; the
-// site term added straight onto -acc / 2: 2910 us, but the error rises to 7.5e-15.
+// fields of 24^4, the call, 3600 -> 3280 us (3000 with the pairs dealt out as in launch_dslash_dw), five of
+// 8x16x8x24 184 -> 168 us, two of 16^3 x 32 271 -> 278 us; error against 64 bits 5.8e-15 both.  Before the pairs
+// were dealt out: the accumulators parked in shared memory during the site term 3410 us; four CTAs per SM (spills)
+// 3530 us; the site term added straight onto -acc / 2 2910 us, but the error rises to 7.5e-15.
 // The loop over the eight directions is rolled (one hop is about 10 KB of code) with the spin structure as
 // run-time selects and sign flips on the integer pipe.  FP64 instructions issue at 1/64 of the FP32 rate,
 // conversions included: y - acc / 2 is summed in FP32 words and takes one FP64 addition a number (formed in
@@ -233,9 +233,10 @@ __device__ __forceinline__ unsigned sign_im(int p) { return (p & 2) ? 0x80000000
 
 template <bool OUT_DW>
 __global__ void __launch_bounds__(128, 3) dslash_dw_pair_kernel(Geom g, const float4* __restrict__ U, const float2* __restrict__ clov,
-                                                                const cplx<float>* __restrict__ in, void* __restrict__ outp, int nrhs) {
-    const int r0 = 2 * (blockIdx.y * blockDim.y + threadIdx.y);
-    const int lane = threadIdx.x, s = lane >> 4, i = blockIdx.x * 16 + (lane & 15);  // V is a multiple of 16
+                                                                const cplx<float>* __restrict__ in, void* __restrict__ outp, int nrhs,
+                                                                int rows) {
+    const int r0 = 2 * (blockIdx.x % rows * blockDim.y + threadIdx.y);
+    const int lane = threadIdx.x, s = lane >> 4, i = blockIdx.x / rows * 16 + (lane & 15);  // V is a multiple of 16
     if (r0 >= nrhs) return;  // (a whole warp)
     const bool two = r0 + 1 < nrhs;  // an odd batch computes its last right-hand side twice and stores it once
     const size_t V = g.V, o0 = (size_t)r0 * 12 * V, o1 = o0 + (two ? 12 * V : 0);
@@ -365,10 +366,13 @@ __global__ void __launch_bounds__(128, 3) dslash_dw_pair_kernel(Geom g, const fl
 int launch_dslash_dw(const Geom& g, const float4* U, const float2* clov, const cplx<float>* in, void* out, bool out_dw, int nrhs,
                      cudaStream_t st) {
     if (nrhs >= 2) {
-        const int pairs = (nrhs + 1) / 2, ry = std::min(pairs, 4);
-        const dim3 grid((unsigned)(g.V / 16), (unsigned)ceil_div(pairs, ry)), block(32, ry);
-        if (out_dw) dslash_dw_pair_kernel<true><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
-        else dslash_dw_pair_kernel<false><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
+        // pairs dealt out evenly to CTAs of up to four, the CTAs of the same sites one after another: six pairs as
+        // 4 + 2 in separate grid rows left half of the second row's warps idle and read the operator twice
+        // (12 fields of 24^4, the call: 3270 -> 3000 us; DRAM reads of the kernel 1.97 GB with the rows apart, 0.76 GB needed)
+        const int pairs = (nrhs + 1) / 2, rows = ceil_div(pairs, 4), ry = ceil_div(pairs, rows);
+        const dim3 grid((unsigned)(g.V / 16) * (unsigned)rows), block(32, ry);
+        if (out_dw) dslash_dw_pair_kernel<true><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs, rows);
+        else dslash_dw_pair_kernel<false><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs, rows);
         DD_CHECK_LAUNCH();
         return 0;
     }
