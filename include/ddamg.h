@@ -348,10 +348,12 @@ void ddamg_debug_fail_allocs(int n);
  * V-cycle precision (FP64 on DOUBLE handles, FP32 on SINGLE and HALF handles, with FP32 copies of
  * D_1, P_1, D_2 and the inverses).  HALF handles also keep FP16 copies: the level-1 SAP reads D_1 and
  * its even inverses in FP16 (the vectors enter in FP32, or as FP16 hi + lo pairs on the tensor cores,
+ * scaled by a power of two per block and field so that a field may have any size that FP32 holds,
  * with FP32 accumulation), and the coarsest level's GMRES and ddamg_ml_apply_D2
  * apply D_2 (and its even inverses) from FP16 tensor-core fragments, with each right-hand-side entry
  * entering as an FP16 hi + lo pair so that the product is the FP16-rounded matrix times the FP32
- * vector to about 2^-22 (2 n_vec1 divisible by 8; otherwise FP32).  The third level is tied to the coarse operator it was built
+ * vector to about 2^-22 (2 n_vec1 divisible by 8; otherwise FP32).  These pairs are not scaled: entries
+ * up to 65504, with an absolute resolution of 2^-36.  The third level is tied to the coarse operator it was built
  * from: after ddamg_run_setup, ddamg_setup_from_vectors or ddamg_set_mass the calls below return
  * DDAMG_ERR_NOT_READY until ddamg_ml_build runs again.
  * Level-1 vectors use the coarse layout of ddamg_restrict ([n_rhs][coarse sites lex][2N]);

@@ -9,6 +9,12 @@
 // and the MR updates stay in registers; only the staged (hi, lo) vectors of the block's sites, 1.3 KB a
 // site and group at nc = 40, go through shared memory.
 //
+// The step is linear in (b, z), and FP16 covers 2^-36 (the low part's last bit) to 2^16 only, so every vector is
+// multiplied by a power of two before it is split and the product divided by it: z by one per site and right-hand
+// side, found as the neighbours are read; everything after the residual by one per block and right-hand side,
+// which brings the largest entry of r to 2^-4 and leaves x_o and the even vectors 2^19 to grow.  The result is
+// that of FP32 vectors at any size of the fields.
+//
 // Matrix blocks are stored in fragment order and go straight from L2 to registers, 16 bytes a lane; a
 // block is used once per product and warp, so shared memory would not save a read.  G groups of four
 // right-hand sides share a CTA (and its L1) when there are enough blocks to fill the chip; with fewer
@@ -42,6 +48,11 @@ __device__ __forceinline__ void mma_k8(float (&d)[4], const uint2& a, unsigned b
                  : "r"(a.x), "r"(a.y), "r"(b0));
 }
 __device__ __forceinline__ unsigned h2u(__half2 v) { return *reinterpret_cast<unsigned*>(&v); }
+// exponent of m >= 0 within -120 .. 120 (zero and subnormal numbers: -120), and 2^e for |e| <= 126
+__device__ __forceinline__ int exponent_of(float m) { return max(-120, min(120, (int)(__float_as_uint(m) >> 23) - 127)); }
+__device__ __forceinline__ float pow2(int e) { return __int_as_float((e + 127) << 23); }
+constexpr int kTop = -4;  // scaled vectors start with their largest entry in [2^kTop, 2^(kTop + 1))
+
 // two values as packed hi and lo halves
 __device__ __forceinline__ void split2(float a, float b, unsigned& hi, unsigned& lo) {
     const __half2 h = __floats2half2_rn(a, b);
@@ -66,6 +77,12 @@ struct Acc {
         for (int m = 0; m < U; ++m)
 #pragma unroll
             for (int i = 0; i < 4; ++i) hi[m][i] = lo[m][i] = 0.f;
+    }
+    __device__ __forceinline__ void scale(float f) {
+#pragma unroll
+        for (int m = 0; m < U; ++m)
+#pragma unroll
+            for (int i = 0; i < 4; ++i) hi[m][i] *= f, lo[m][i] *= f;
     }
     __device__ __forceinline__ float at(int m, int i) const { return fmaf(lo[m][i], 1.f / kSplit, hi[m][i]); }
     // the complex rows 8 q + g of right-hand side t
@@ -106,10 +123,11 @@ __device__ __forceinline__ void times_staged(Acc<U>& acc, const unsigned char* B
         }
     }
 }
-// acc += B x for the vector x read from global memory: xr = this lane's right-hand side (column g >> 1) at the
-// site, part = g & 1 (real or imaginary), on = false: zero
+// acc += 2^(kTop - ex) B x for the vector x read from global memory: xr = this lane's right-hand side (column
+// g >> 1) at the site, part = g & 1 (real or imaginary), on = false: zero.  ex, the exponent that the right-hand
+// side's x is scaled by, rises when an entry exceeds it by more than 2^8; acc then moves to the new scale.
 template <int U>
-__device__ __forceinline__ void times_global(Acc<U>& acc, const unsigned char* B, const cplx<float>* xr, int part, bool on, int lane) {
+__device__ __forceinline__ void times_global(Acc<U>& acc, int& ex, const unsigned char* B, const cplx<float>* xr, int part, bool on, int lane) {
     using F = Frag<U>;
     const int t = lane & 3;
     float4 v[U];  // entries 8 j + 2 t, 8 j + 2 t + 1
@@ -118,9 +136,20 @@ __device__ __forceinline__ void times_global(Acc<U>& acc, const unsigned char* B
         v[j] = make_float4(0.f, 0.f, 0.f, 0.f);
         if (on) v[j] = *reinterpret_cast<const float4*>(xr + 8 * j + 2 * t);
     }
+    float m = 0.f;
+#pragma unroll
+    for (int j = 0; j < U; ++j) m = fmaxf(fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y))), fmaxf(fabsf(v[j].z), fabsf(v[j].w)));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
+    m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
+    const int e = exponent_of(m), up = e > ex + 8 ? e - ex : 0;
+    if (__any_sync(0xffffffffu, up)) {
+        ex += up;
+        acc.scale(pow2(-min(126, __shfl_sync(0xffffffffu, up, 8 * t))));  // (lane 8 t: a lane of column 2 t)
+    }
+    const float f = pow2(kTop - ex);
     unsigned b[U], c[U];
 #pragma unroll
-    for (int j = 0; j < U; ++j) split2(part ? v[j].y : v[j].x, part ? v[j].w : v[j].z, b[j], c[j]);
+    for (int j = 0; j < U; ++j) split2(f * (part ? v[j].y : v[j].x), f * (part ? v[j].w : v[j].z), b[j], c[j]);
 #pragma unroll
     for (int kt = 0; kt < F::KT; ++kt)
 #pragma unroll
@@ -198,17 +227,24 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
     // y = r at site c: b - D_k z (z of out-of-block neighbours belongs to the other colour, not written here)
     auto residual = [&](int c) {
         acc.zero();
+        int ex = -120;
         const bool on = (g >> 1) < nr;
         const cplx<float>* zr = z + (size_t)(r0 + (on ? g >> 1 : 0)) * fs;
 #pragma unroll 1
         for (int d = 0; d < 9; ++d) {
             const int n = d == 0 ? c : __ldg(v.nbr1 + (size_t)(d - 1) * NB + c);
-            times_global<U>(acc, blk(c, d), zr + (size_t)n * F::NC, g & 1, on, lane);
+            times_global<U>(acc, ex, blk(c, d), zr + (size_t)n * F::NC, g & 1, on, lane);
         }
         acc.rows(y);
+        const float f = pow2(__shfl_sync(0xffffffffu, ex, 8 * t) - kTop);
         const cplx<float>* br = b + (size_t)(r0 + (t < nr ? t : 0)) * fs + (size_t)c * F::NC + g;
 #pragma unroll
-        for (int q = 0; q < U; ++q) y[q] = t < nr ? br[8 * q] - y[q] : czero<float>();
+        for (int q = 0; q < U; ++q) y[q] = t < nr ? br[8 * q] - f * y[q] : czero<float>();
+    };
+    float big = 0.f;  // largest entry of r on this warp's sites, of right-hand side t
+    auto note = [&]() {
+#pragma unroll
+        for (int q = 0; q < U; ++q) big = fmaxf(big, fmaxf(fabsf(y[q].re), fabsf(y[q].im)));
     };
     // acc += sum of the in-block hops of the staged field X (sites of the other parity, local indices from l0)
     auto hops = [&](int l, int c, const __half* X, int l0) {
@@ -228,18 +264,30 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
         acc.rows(y);
     };
     residual(ce);
+    note();
+#pragma unroll
+    for (int q = 0; q < U; ++q) own[q * 32] = y[q];  // r_e
+    residual(co);
+    note();
+#pragma unroll
+    for (int o = 4; o < 32; o <<= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+    if (g == 0) red[s * 4 + t] = big;
+    sync();
+    for (int q = 0; q < He; ++q) big = fmaxf(big, red[q * 4 + t]);
+    // from here on the block's vectors are 2^(kTop - ex) times r and x
+    const int ex = exponent_of(big);
+    const float down = pow2(kTop - ex);
 #pragma unroll
     for (int q = 0; q < U; ++q) {
-        own[q * 32] = y[q];  // r_e
+        rho[q] = down * y[q];
+        y[q] = down * own[q * 32];
+        own[q * 32] = y[q];
         own[(U + q) * 32] = czero<float>();
     }
     inv_even();
     stage<U>(XE + (size_t)s * F::SLOT, y, -1.f, lane);
-    residual(co);
     sync();
     // rho = r_o - A_oe A_ee^{-1} r_e
-#pragma unroll
-    for (int q = 0; q < U; ++q) rho[q] = y[q];
     acc.zero();
     hops(He + s, co, XE, 0);
     acc.rows(y);
@@ -300,13 +348,14 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
     for (int q = 0; q < U; ++q) y[q] = y[q] + own[q * 32];
     inv_even();
     if (t < nr) {
+        const float f = pow2(ex - kTop);
         cplx<float>* ze = z + (size_t)(r0 + t) * fs + (size_t)ce * F::NC + g;
         cplx<float>* zo = z + (size_t)(r0 + t) * fs + (size_t)co * F::NC + g;
         cplx<float> u[U], w[U];
 #pragma unroll
         for (int q = 0; q < U; ++q) u[q] = ze[8 * q], w[q] = zo[8 * q];
 #pragma unroll
-        for (int q = 0; q < U; ++q) ze[8 * q] = u[q] + y[q], zo[8 * q] = w[q] + own[(U + q) * 32];
+        for (int q = 0; q < U; ++q) ze[8 * q] = u[q] + f * y[q], zo[8 * q] = w[q] + f * own[(U + q) * 32];
     }
 }
 

@@ -231,3 +231,38 @@ def test_half_prolongation_by_block_and_right_hand_sides(dims, block, n_vec, nrh
     for r in range(nrhs):
         ref = agg.prolong(e[r])
         assert np.max(np.abs(np.reshape(got[r], ref.shape) - ref)) <= 4e-3 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("dims,n_vec,block1,mr", [((8, 8, 8, 8), 8, (2, 2, 2, 2), 4), ((8, 8, 8, 8), 16, (2, 2, 2, 2), 1),
+                                                  ((8, 8, 8, 8), 20, (2, 2, 2, 2), 4), ((8, 8, 8, 8), 24, (2, 2, 2, 1), 4),
+                                                  ((8, 8, 8, 16), 8, (2, 2, 2, 4), 0)])
+def test_level1_sap_of_fields_of_very_different_size(dims, n_vec, block1, mr):
+    """The half-precision level-1 SAP is homogeneous in its right-hand side: fields from 1e-30 to 1e30, a zero
+    field and a field that is tiny on all sites but one, each to the 1e-5 of its own result's maximum that
+    test_level1_sap_on_tensor_cores derives; level-1 blocks of 8, 16 and 32 sites, 0, 1 and 4 MR steps."""
+    from oracle.lattice import Lattice
+    from oracle.multilevel import StencilOperator, StencilSAP
+    from paper_1303_1377_gb300 import ddamg
+
+    l1 = tuple(d // 2 for d in dims)
+    nb = int(np.prod(l1))
+    s, _ = _solver(dims, n_vec=n_vec, block=(2, 2, 2, 2), precision=ddamg.PREC_HALF)
+    x = synth.gaussian_coarse(nb, 2 * n_vec, 7, seed=35)
+    x[:5] *= 10.0 ** np.array([-30, -12, 6, 20, 30])[:, None, None]
+    x[5] = 0
+    x[6, 1:] *= 1e-12
+    with s:
+        s.setup_from_vectors(synth.random_test_vectors(dims, n_vec, seed=31))
+        s.ml_build(synth.gaussian_coarse(nb, 2 * n_vec, 3, seed=32), ddamg.ml_default_params(n_vec1=3, block1=block1, mr_steps1=mr))
+        B = s.coarse_stencil()
+        got = s.ml_apply_sap1(x, 2)
+
+    def r16(v):
+        return v.real.astype(np.float32).astype(np.float16) + 1j * v.imag.astype(np.float32).astype(np.float16).astype(np.float64)
+
+    sap = StencilSAP(StencilOperator(Lattice(l1), r16(B)), block1, mr_steps=mr)
+    inv = r16(np.linalg.inv(B[:, 0]))
+    sap.apply_Aee_inv = lambda f: np.einsum("xij,xj->xi", inv, f)
+    for r in range(7):
+        ref = sap.apply(x[r], 2)
+        assert np.max(np.abs(got[r] - ref)) <= 1e-5 * np.max(np.abs(ref))
