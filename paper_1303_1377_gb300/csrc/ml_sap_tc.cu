@@ -4,14 +4,16 @@
 // The unit of work is one warp per (even/odd site pair of the block, four right-hand sides).  A product
 // B x of an nc x nc block with the four right-hand sides is a real product [Re B; Im B] (2 nc rows) times
 // [Re x_r, Im x_r interleaved] (8 columns): U = nc / 8 m-tiles of mma.sync with K = nc.  The vector enters
-// as two FP16 numbers, hi + 2^-11 lo, so that the product is the FP16-stored matrix times x to about 2^-22
-// with FP32 accumulation.  A lane ends with the complex rows 8 q + g of one right-hand side, so rho, x_o
+// as two FP16 numbers, hi + 2^-11 lo, so that the product is the FP16-stored matrix times x to about 2^-22.
+// The tensor cores' FP32 accumulation truncates, so every product starts from zero and is added to the running
+// sum in FP32 registers: with the accumulators kept over the nine products of a row the error grew to 1.35 times
+// that of FP32 vectors on the CUDA cores (8.9e-7 against 6.6e-7 rms at nc = 40; now 1.4e-7).  A lane ends with the complex rows 8 q + g of one right-hand side, so rho, x_o
 // and the MR updates stay in registers; only the staged (hi, lo) vectors of the block's sites, 1.3 KB a
 // site and group at nc = 40, go through shared memory.
 //
 // The step is linear in (b, z), and FP16 covers 2^-36 (the low part's last bit) to 2^16 only, so every vector is
-// multiplied by a power of two before it is split and the product divided by it: z by one per site and right-hand
-// side, found as the neighbours are read; everything after the residual by one per block and right-hand side,
+// multiplied by a power of two before it is split and the product divided by it: z by one per site read and
+// right-hand side; everything after the residual by one per block and right-hand side,
 // which brings the largest entry of r to 2^-4 and leaves x_o and the even vectors 2^19 to grow.  The result is
 // that of FP32 vectors at any size of the fields.
 //
@@ -21,8 +23,8 @@
 // blocks each group is its own CTA.  mma.sync rather than tcgen05: a product has 80 rows and 8 columns
 // per site, each site has its own matrix, and the result feeds the next product of the chain.
 //
-// 12 right-hand sides, one colour: 32^4 (128 level-1 blocks of 2^4 sites, nc = 40) 531 -> 150 us, 32x16^3 (16
-// blocks) 519 -> 62 us; before, one thread per row on the CUDA cores.
+// 12 right-hand sides, nu = 2, the call: 32^4 (128 level-1 blocks of 2^4 sites, nc = 40) 2244 -> 645 us, a colour
+// from 531 us with one thread per row on the CUDA cores; 16 blocks 249 us.
 #include <algorithm>
 
 #include <cuda_fp16.h>
@@ -78,19 +80,14 @@ struct Acc {
 #pragma unroll
             for (int i = 0; i < 4; ++i) hi[m][i] = lo[m][i] = 0.f;
     }
-    __device__ __forceinline__ void scale(float f) {
-#pragma unroll
-        for (int m = 0; m < U; ++m)
-#pragma unroll
-            for (int i = 0; i < 4; ++i) hi[m][i] *= f, lo[m][i] *= f;
-    }
     __device__ __forceinline__ float at(int m, int i) const { return fmaf(lo[m][i], 1.f / kSplit, hi[m][i]); }
-    // the complex rows 8 q + g of right-hand side t
-    __device__ __forceinline__ void rows(cplx<float> (&y)[U]) const {
+    // y += f times the complex rows 8 q + g of right-hand side t
+    __device__ __forceinline__ void add_rows(cplx<float> (&y)[U], float f = 1.f) const {
 #pragma unroll
         for (int q = 0; q < U; ++q) {
             const int a = q >> 1, i = 2 * (q & 1), b = (q + U) >> 1, j = 2 * ((q + U) & 1);
-            y[q] = mk(at(a, i) - at(b, j + 1), at(b, j) + at(a, i + 1));
+            y[q].re = fmaf(f, at(a, i) - at(b, j + 1), y[q].re);
+            y[q].im = fmaf(f, at(b, j) + at(a, i + 1), y[q].im);
         }
     }
 };
@@ -124,8 +121,7 @@ __device__ __forceinline__ void times_staged(Acc<U>& acc, const unsigned char* B
     }
 }
 // acc += 2^(kTop - ex) B x for the vector x read from global memory: xr = this lane's right-hand side (column
-// g >> 1) at the site, part = g & 1 (real or imaginary), on = false: zero.  ex, the exponent that the right-hand
-// side's x is scaled by, rises when an entry exceeds it by more than 2^8; acc then moves to the new scale.
+// g >> 1) at the site, part = g & 1 (real or imaginary), on = false: zero; ex = the exponent of its largest entry
 template <int U>
 __device__ __forceinline__ void times_global(Acc<U>& acc, int& ex, const unsigned char* B, const cplx<float>* xr, int part, bool on, int lane) {
     using F = Frag<U>;
@@ -141,11 +137,7 @@ __device__ __forceinline__ void times_global(Acc<U>& acc, int& ex, const unsigne
     for (int j = 0; j < U; ++j) m = fmaxf(fmaxf(m, fmaxf(fabsf(v[j].x), fabsf(v[j].y))), fmaxf(fabsf(v[j].z), fabsf(v[j].w)));
     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 1));
     m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, 2));
-    const int e = exponent_of(m), up = e > ex + 8 ? e - ex : 0;
-    if (__any_sync(0xffffffffu, up)) {
-        ex += up;
-        acc.scale(pow2(-min(126, __shfl_sync(0xffffffffu, up, 8 * t))));  // (lane 8 t: a lane of column 2 t)
-    }
+    ex = exponent_of(m);
     const float f = pow2(kTop - ex);
     unsigned b[U], c[U];
 #pragma unroll
@@ -224,22 +216,26 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
     const int ce = site[s], co = site[He + s];  // this warp's even and odd site
     Acc<U> acc;
     cplx<float> y[U], rho[U];
+    auto clear = [](cplx<float> (&v)[U]) {
+#pragma unroll
+        for (int q = 0; q < U; ++q) v[q] = czero<float>();
+    };
     // y = r at site c: b - D_k z (z of out-of-block neighbours belongs to the other colour, not written here)
     auto residual = [&](int c) {
-        acc.zero();
-        int ex = -120;
+        clear(y);
         const bool on = (g >> 1) < nr;
         const cplx<float>* zr = z + (size_t)(r0 + (on ? g >> 1 : 0)) * fs;
 #pragma unroll 1
         for (int d = 0; d < 9; ++d) {
             const int n = d == 0 ? c : __ldg(v.nbr1 + (size_t)(d - 1) * NB + c);
+            int ex;
+            acc.zero();
             times_global<U>(acc, ex, blk(c, d), zr + (size_t)n * F::NC, g & 1, on, lane);
+            acc.add_rows(y, pow2(__shfl_sync(0xffffffffu, ex, 8 * t) - kTop));
         }
-        acc.rows(y);
-        const float f = pow2(__shfl_sync(0xffffffffu, ex, 8 * t) - kTop);
         const cplx<float>* br = b + (size_t)(r0 + (t < nr ? t : 0)) * fs + (size_t)c * F::NC + g;
 #pragma unroll
-        for (int q = 0; q < U; ++q) y[q] = t < nr ? br[8 * q] - f * y[q] : czero<float>();
+        for (int q = 0; q < U; ++q) y[q] = t < nr ? br[8 * q] - y[q] : czero<float>();
     };
     float big = 0.f;  // largest entry of r on this warp's sites, of right-hand side t
     auto note = [&]() {
@@ -247,11 +243,15 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
         for (int q = 0; q < U; ++q) big = fmaxf(big, fmaxf(fabsf(y[q].re), fabsf(y[q].im)));
     };
     // acc += sum of the in-block hops of the staged field X (sites of the other parity, local indices from l0)
-    auto hops = [&](int l, int c, const __half* X, int l0) {
+    auto hops = [&](cplx<float> (&v)[U], int l, int c, const __half* X, int l0) {
 #pragma unroll 1
         for (int d = 0; d < 8; ++d) {
             const int n = nbl[l * 8 + d];
-            if (n >= 0) times_staged<U>(acc, blk(c, 1 + d), X + (size_t)(n - l0) * F::SLOT, lane);
+            if (n >= 0) {
+                acc.zero();
+                times_staged<U>(acc, blk(c, 1 + d), X + (size_t)(n - l0) * F::SLOT, lane);
+                acc.add_rows(v);
+            }
         }
     };
     // y <- D_ee^{-1} y on the even site
@@ -261,7 +261,8 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
         __syncwarp();
         acc.zero();
         times_staged<U>(acc, Dm + (size_t)ce * F::BYTES, XU, lane);
-        acc.rows(y);
+        clear(y);
+        acc.add_rows(y);
     };
     residual(ce);
     note();
@@ -288,28 +289,23 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
     stage<U>(XE + (size_t)s * F::SLOT, y, -1.f, lane);
     sync();
     // rho = r_o - A_oe A_ee^{-1} r_e
-    acc.zero();
-    hops(He + s, co, XE, 0);
-    acc.rows(y);
+    hops(rho, He + s, co, XE, 0);
 #pragma unroll
-    for (int q = 0; q < U; ++q) {
-        rho[q] = rho[q] + y[q];
-        y[q] = mr_steps > 0 ? rho[q] : czero<float>();
-    }
+    for (int q = 0; q < U; ++q) y[q] = mr_steps > 0 ? rho[q] : czero<float>();
     stage<U>(XO + (size_t)s * F::SLOT, y, 1.f, lane);
     sync();
 #pragma unroll 1
     for (int it = 0; it < mr_steps; ++it) {
-        acc.zero();  // t_e = A_ee^{-1} A_eo rho, staged with the sign it enters S rho with
-        hops(s, ce, XO, He);
-        acc.rows(y);
+        clear(y);  // t_e = A_ee^{-1} A_eo rho, staged with the sign it enters S rho with
+        hops(y, s, ce, XO, He);
         inv_even();
         stage<U>(XE + (size_t)s * F::SLOT, y, -1.f, lane);
         sync();
-        acc.zero();  // S rho = A_oo rho - A_oe t_e
+        clear(y);  // S rho = A_oo rho - A_oe t_e
+        acc.zero();
         times_staged<U>(acc, blk(co, 0), XO + (size_t)s * F::SLOT, lane);
-        hops(He + s, co, XE, 0);
-        acc.rows(y);
+        acc.add_rows(y);
+        hops(y, He + s, co, XE, 0);
         float nre = 0.f, nim = 0.f, den = 0.f;
 #pragma unroll
         for (int q = 0; q < U; ++q) {
@@ -341,11 +337,9 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
         sync();
     }
     // x_e = A_ee^{-1} (r_e - A_eo x_o); z += x on the block
-    acc.zero();
-    hops(s, ce, XO, He);
-    acc.rows(y);
 #pragma unroll
-    for (int q = 0; q < U; ++q) y[q] = y[q] + own[q * 32];
+    for (int q = 0; q < U; ++q) y[q] = own[q * 32];
+    hops(y, s, ce, XO, He);
     inv_even();
     if (t < nr) {
         const float f = pow2(ex - kTop);
@@ -412,9 +406,12 @@ template <int U>
 static int launch_u(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps, cudaStream_t st) {
     // Three groups per CTA read each matrix block once from L2 (12 fields, 128 blocks of nc = 40: 150 us a
     // colour against 169 us with one group per CTA); one group per CTA spreads few blocks over more SMs
-    // (16 blocks: 62 against about 134 us).  The line is one CTA per SM at one group each.
+    // (16 blocks: 62 against about 134 us).  The line is one CTA per SM at one group each.  At nc = 48 the 80
+    // registers of the wide form spill (blocks of 8 sites, the call: 826 us with one group, 996 us with three).
     const bool wide = v.Vb1e <= 8 && nrhs > 4 && (long long)(v.NB2 / 2) * ceil_div(nrhs, 4) > 152;
-    return wide ? launch_ug<U, 3>(v, b, z, nrhs, colour, mr_steps, st) : launch_ug<U, 1>(v, b, z, nrhs, colour, mr_steps, st);
+    if constexpr (U < 6)
+        if (wide) return launch_ug<U, 3>(v, b, z, nrhs, colour, mr_steps, st);
+    return launch_ug<U, 1>(v, b, z, nrhs, colour, mr_steps, st);
 }
 int launch_ml_sap_tc(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps, cudaStream_t st) {
     switch (v.nc / 8) {

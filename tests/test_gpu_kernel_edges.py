@@ -266,3 +266,33 @@ def test_level1_sap_of_fields_of_very_different_size(dims, n_vec, block1, mr):
     for r in range(7):
         ref = sap.apply(x[r], 2)
         assert np.max(np.abs(got[r] - ref)) <= 1e-5 * np.max(np.abs(ref))
+
+
+@pytest.mark.parametrize("n_vec", [8, 12, 20])
+def test_level1_sap_on_tensor_cores_is_as_accurate_as_in_fp32(n_vec):
+    """The same level-1 SAP on a SINGLE handle (FP32 operator, vectors and accumulation on the CUDA cores) sets the
+    bound: the half-precision handle's error against 64 bits on the operator as it stores it is no larger."""
+    from oracle.lattice import Lattice
+    from oracle.multilevel import StencilOperator, StencilSAP
+    from paper_1303_1377_gb300 import ddamg
+
+    def r32(v):
+        return v.astype(np.complex64).astype(np.complex128)
+
+    def r16(v):
+        return v.real.astype(np.float32).astype(np.float16) + 1j * v.imag.astype(np.float32).astype(np.float16).astype(np.float64)
+
+    dims, err = (8, 8, 8, 8), {}
+    x = synth.gaussian_coarse(256, 2 * n_vec, 6, seed=33)
+    for prec, stored in ((ddamg.PREC_SINGLE, r32), (ddamg.PREC_HALF, r16)):
+        s, _ = _solver(dims, n_vec=n_vec, block=(2, 2, 2, 2), precision=prec)
+        with s:
+            s.setup_from_vectors(synth.random_test_vectors(dims, n_vec, seed=31))
+            s.ml_build(synth.gaussian_coarse(256, 2 * n_vec, 3, seed=32), ddamg.ml_default_params(n_vec1=3))
+            B = s.coarse_stencil()
+            got = s.ml_apply_sap1(x, 2)
+        sap = StencilSAP(StencilOperator(Lattice((4, 4, 4, 4)), stored(B)), (2, 2, 2, 2), mr_steps=4)
+        inv = stored(np.linalg.inv(B[:, 0]))
+        sap.apply_Aee_inv = lambda f: np.einsum("xij,xj->xi", inv, f)
+        err[prec] = np.linalg.norm(got - np.stack([sap.apply(x[r], 2) for r in range(6)]))
+    assert err[ddamg.PREC_HALF] <= err[ddamg.PREC_SINGLE]
