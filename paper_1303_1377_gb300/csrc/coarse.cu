@@ -8,6 +8,7 @@
 // Vectors: cplx[nrhs][sites][nc] addressed through (pointer, rhs stride,
 // first site) so that half vectors and full vectors share one kernel.
 #include <algorithm>
+#include <type_traits>
 
 #include "kernels.h"
 
@@ -35,13 +36,13 @@ __device__ __forceinline__ void load_pair(const double* p, cplx<double>& a, cplx
 
 // acc[2][NRP] += sum over columns q in [q0, q1) of M(q)[2p..2p+1] * xs[q][0..NRP);
 // column q of the stacked matrices starts at first + q * nc complex entries (slots are
-// contiguous nc x nc column-major blocks).
-template <typename T, typename S, int NRP>
+// contiguous nc x nc column-major blocks).  UNR columns are in flight.
+template <typename T, typename S, int NRP, int UNR>
 __device__ __forceinline__ void gemm_slice(const S* first, int nc, int p, int q0, int q1, const cplx<T>* xs,
                                            cplx<T> (&acc)[2][NRP]) {
     const S* bp = first + 2 * ((size_t)q0 * nc + 2 * p);
     const cplx<T>* xq = xs + (size_t)q0 * NRP;
-#pragma unroll(NRP == 1 ? 4 : 2)
+#pragma unroll(UNR)
     for (int q = q0; q < q1; ++q, bp += 2 * nc, xq += NRP) {
         cplx<T> b0, b1;
         load_pair(bp, b0, b1);
@@ -61,7 +62,7 @@ __device__ __forceinline__ void gemm_slice(const S* first, int nc, int p, int q0
 // WIDE (few sites, one or two right-hand sides): 1024 threads per CTA.  Such a launch is bound by the latency of
 // the matrix columns a thread reads one after the other (60 of them at 2N = 40 with 128 threads, 8 with 1024),
 // and there are not enough sites for more CTAs.
-template <typename T, typename S, int NRP, bool WIDE>
+template <typename T, typename S, int NRP, bool WIDE, int UNR>
 __global__ void __launch_bounds__(WIDE ? 1024 : 128) coarse_stencil_kernel(CoarseOp<S> op, int site_begin, CVec<T> xin, CVec<T> xself,
                                                              int self_mode, T hop_sign, int apply_inv, CVec<T> out, int nrhs) {
     extern __shared__ unsigned char smem_raw[];
@@ -124,7 +125,7 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 128) coarse_stencil_kernel(Coars
             }
         }
     };
-    if (act && nslots > 0) gemm_slice<T, S, NRP>(first, nc, p, (g * Kt) / KG, ((g + 1) * Kt) / KG, xs, acc);
+    if (act && nslots > 0) gemm_slice<T, S, NRP, UNR>(first, nc, p, (g * Kt) / KG, ((g + 1) * Kt) / KG, xs, acc);
     __syncthreads();
     // reduce the KG partial sums: red[g][row][r]
     cplx<T>* red = xs;
@@ -144,7 +145,7 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 128) coarse_stencil_kernel(Coars
         for (int h = 0; h < 2; ++h)
 #pragma unroll
             for (int r = 0; r < NRP; ++r) acc[h][r] = czero<T>();
-        if (act) gemm_slice<T, S, NRP>(dfirst, nc, p, (g * nc) / KG, ((g + 1) * nc) / KG, vsum, acc);
+        if (act) gemm_slice<T, S, NRP, UNR>(dfirst, nc, p, (g * nc) / KG, ((g + 1) * nc) / KG, vsum, acc);
         __syncthreads();
         if (act)
 #pragma unroll
@@ -162,7 +163,7 @@ __global__ void __launch_bounds__(WIDE ? 1024 : 128) coarse_stencil_kernel(Coars
     }
 }
 
-template <typename T, typename S, int NRP, bool WIDE>
+template <typename T, typename S, int NRP, bool WIDE, int UNR>
 static int launch_stencil_threads(const CoarseOp<S>& op, int site_begin, int nsites, CVec<T> xin, CVec<T> xself, int self_mode,
                                   T hop_sign, int apply_inv, CVec<T> out, int nrhs, cudaStream_t st) {
     const int RP = op.nc / 2;
@@ -174,25 +175,41 @@ static int launch_stencil_threads(const CoarseOp<S>& op, int site_begin, int nsi
     size_t smem = stage > reduce ? stage : reduce;
     // set once per kernel instance (a function-local static initialiser is thread safe)
     static const bool attr = [] {
-        cudaFuncSetAttribute(coarse_stencil_kernel<T, S, NRP, WIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
+        cudaFuncSetAttribute(coarse_stencil_kernel<T, S, NRP, WIDE, UNR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
         return true;
     }();
     (void)attr;
-    coarse_stencil_kernel<T, S, NRP, WIDE><<<nsites, nt, smem, st>>>(op, site_begin, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs);
+    coarse_stencil_kernel<T, S, NRP, WIDE, UNR><<<nsites, nt, smem, st>>>(op, site_begin, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs);
     DD_CHECK_LAUNCH();
     return 0;
 }
 template <typename T, typename S, int NRP>
 static int launch_stencil_nrp(const CoarseOp<S>& op, int site_begin, int nsites, CVec<T> xin, CVec<T> xself, int self_mode,
                               T hop_sign, int apply_inv, CVec<T> out, int nrhs, cudaStream_t st) {
-    // FP32, 2N = 40, us per launch wide / narrow: one right-hand side 9.3 / 17.0 (8 sites), 9.9 / 17.9 (128), 11.5 /
+    auto run = [&](auto wide, auto unr) {
+        return launch_stencil_threads<T, S, NRP, decltype(wide)::value, decltype(unr)::value>(op, site_begin, nsites, xin, xself, self_mode,
+                                                                                              hop_sign, apply_inv, out, nrhs, st);
+    };
+    using Two = std::integral_constant<int, 2>;
+    using Four = std::integral_constant<int, 4>;
+    constexpr int kSM = 152;
+    // WIDE.  FP32, 2N = 40, us per launch wide / narrow: one right-hand side 9.3 / 17.0 (8 sites), 9.9 / 17.9 (128), 11.5 /
     // 18.0 (256); two 11.3 / 14.0 (8), 11.4 / 14.3 (128), 17.0 / 14.9 (256); four 14.8 / 16.2 (8), 25.6 / 18.6 (256).
-    // FP64: one 27.7 / 30.9 (128), two 44.9 / 44.6.
-    if constexpr (NRP == 1 || (NRP == 2 && sizeof(T) == 4)) {
-        if (nsites <= 152 * (NRP == 1 ? 2 : 1))
-            return launch_stencil_threads<T, S, NRP, true>(op, site_begin, nsites, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs, st);
+    // FP64, one right-hand side, 128 sites 27.7 / 30.9; 256 sites, the call: 2N = 16 55 / 51, 40 80 / 77, 48 93 / 97, 56
+    // 108 / 142 (long columns only); two right-hand sides, 128 sites 44.9 / 44.6.
+    if constexpr (NRP == 1) {
+        if (nsites <= kSM || (nsites <= 2 * kSM && (sizeof(T) == 4 || op.nc >= 48))) return run(std::true_type(), Four());
     }
-    return launch_stencil_threads<T, S, NRP, false>(op, site_begin, nsites, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs, st);
+    if constexpr (NRP == 2 && sizeof(T) == 4) {
+        if (nsites <= kSM) return run(std::true_type(), Two());
+    }
+    // One right-hand side, FP32: four columns in flight take 40 registers, 12 CTAs per SM; with more sites than that the
+    // 16 CTAs of two columns in flight are better.  The call, 2N = 56, four / two: 1024 sites 99 / 113 us, 1536 sites
+    // 107 / 119, 2048 sites 162 / 129.
+    if constexpr (NRP == 1) {
+        if (sizeof(T) == 8 || nsites <= 12 * kSM) return run(std::false_type(), Four());
+    }
+    return run(std::false_type(), Two());
 }
 
 // batch of up to kMaxCoarseBatch right-hand sides per launch; larger batches are split

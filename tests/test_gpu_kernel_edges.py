@@ -296,3 +296,22 @@ def test_level1_sap_on_tensor_cores_is_as_accurate_as_in_fp32(n_vec):
         sap.apply_Aee_inv = lambda f: np.einsum("xij,xj->xi", inv, f)
         err[prec] = np.linalg.norm(got - np.stack([sap.apply(x[r], 2) for r in range(6)]))
     assert err[ddamg.PREC_HALF] <= err[ddamg.PREC_SINGLE]
+
+
+@pytest.mark.parametrize("prec,tol", [("DOUBLE", 1e-13), ("SINGLE", 1e-6)])
+@pytest.mark.parametrize("dims,block,n_vec", [((16, 16, 16, 8), (2, 2, 2, 2), 5), ((16, 16, 16, 8), (2, 2, 4, 4), 3),
+                                              ((16, 16, 16, 16), (4, 4, 4, 4), 8), ((16, 16, 16, 16), (4, 4, 4, 4), 24)])
+def test_coarse_stencil_of_one_field_by_sites_and_columns(prec, tol, dims, block, n_vec):
+    """D_c of one field on 256 (short and long columns), 512 and 2048 sites, on both sides of the lines between the forms
+    of the stencil kernel, against the handle's own stencil in FP64, at the stated bounds."""
+    from oracle.lattice import Lattice
+    from oracle.multilevel import StencilOperator
+    from paper_1303_1377_gb300 import ddamg
+
+    s, _ = _solver(dims, n_vec=n_vec, block=block, precision=getattr(ddamg, "PREC_" + prec))
+    with s:
+        s.setup_from_vectors(synth.random_test_vectors(dims, n_vec, seed=91))
+        x = synth.gaussian_coarse(s.n_coarse, s.coarse_dof, 1, seed=92)
+        got, B = s.apply_Dc(x)[0], s.coarse_stencil()
+    ref = StencilOperator(Lattice(tuple(d // b for d, b in zip(dims, block))), B).apply(x[0])
+    assert np.max(np.abs(got - ref)) < tol * np.max(np.abs(ref))
