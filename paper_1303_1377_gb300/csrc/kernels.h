@@ -92,7 +92,7 @@ int launch_restrict_tc(const Geom& g, const cplx<__half>* P, int N, const cplx<f
 bool prolong_tc_supported(const Geom& g, int N);
 int launch_prolong_tc(const Geom& g, const cplx<__half>* P, int N, const cplx<float>* in, cplx<float>* out, int nrhs, cudaStream_t st);
 // the same with the result in FP64 in the caller's layout ([field][site lex[i]][12])
-bool prolong_tc_lex_supported(const Geom& g, int N);
+bool prolong_tc_lex_supported(const Geom& g, int N, int nrhs);
 int launch_prolong_tc_lex(const Geom& g, const cplx<__half>* P, int N, const cplx<float>* in, cplx<double>* out, const int* lex, int nrhs,
                           cudaStream_t st);
 int launch_gram_schmidt(const Geom& g, cplx<double>* P, int N, int* rank_fail, cudaStream_t st);

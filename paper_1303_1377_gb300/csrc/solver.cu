@@ -2147,7 +2147,7 @@ static int prolong_T(ddamg_handle* h, const double* in, double* out, int n_rhs) 
     cplx<T>* o = a + cn * n_rhs;
     DD_TRY(coarse_in<T>(h, in, n_rhs, a));
     if constexpr (std::is_same<T, float>::value) {
-        if (h->half() && prolong_tc_lex_supported(h->g, h->N)) {  // the kernel writes the caller's layout itself
+        if (h->half() && prolong_tc_lex_supported(h->g, h->N, n_rhs)) {  // the kernel writes the caller's layout itself
             void* dv;
             bool host;
             DD_TRY(stage_out_ptr(h->ws_io[1], out, sizeof(cplx<double>) * fld * n_rhs, &dv, &host));

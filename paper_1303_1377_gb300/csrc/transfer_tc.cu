@@ -311,7 +311,13 @@ int launch_restrict_tc(const Geom& g, const cplx<__half>* P, int N, const cplx<f
 
 bool prolong_tc_supported(const Geom& g, int N) { return g.Vb % 16 == 0 && N <= kProKPad; }
 
-bool prolong_tc_lex_supported(const Geom& g, int N) { return prolong_tc_supported(g, N) && g.Vb % kProSites == 0; }
+// Writing the caller's layout keeps a CTA at its aggregate for one more pass over its sites: with few aggregates and
+// several fields the second pass, spread over the chip, is quicker.  us per call, N = 20, the caller's layout / through
+// the internal one: 16 aggregates 2 fields 51 / 54, 4 55 / 54, 8 66 / 60, 12 74 / 62, 24 120 / 90; 32 aggregates 4 55 / 57,
+// 8 66 / 60, 12 75 / 64; 64 aggregates 4 56 / 60, 8 67 / 68, 12 75 / 82; 128 aggregates 12 98 / 103.
+bool prolong_tc_lex_supported(const Geom& g, int N, int nrhs) {
+    return prolong_tc_supported(g, N) && g.Vb % kProSites == 0 && (g.NB >= 64 || nrhs <= 4);
+}
 
 template <bool LEX>
 static int launch_prolong_tc_t(const Geom& g, const cplx<__half>* P, int N, const cplx<float>* in, void* out, const int* lex, int nrhs,

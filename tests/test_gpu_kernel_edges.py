@@ -315,3 +315,18 @@ def test_coarse_stencil_of_one_field_by_sites_and_columns(prec, tol, dims, block
         got, B = s.apply_Dc(x)[0], s.coarse_stencil()
     ref = StencilOperator(Lattice(tuple(d // b for d, b in zip(dims, block))), B).apply(x[0])
     assert np.max(np.abs(got - ref)) < tol * np.max(np.abs(ref))
+
+
+def test_half_prolongation_gives_the_same_bits_by_either_route():
+    """Few aggregates: up to four fields leave the kernel in the caller's layout, larger batches go through the internal
+    one; the same products either way."""
+    from paper_1303_1377_gb300 import ddamg
+
+    dims, n_vec = (8, 8, 8, 8), 8
+    s, _ = _solver(dims, n_vec=n_vec, precision=ddamg.PREC_HALF)
+    with s:
+        s.setup_from_vectors(synth.random_test_vectors(dims, n_vec, seed=75))
+        e = synth.gaussian_coarse(s.n_coarse, s.coarse_dof, 13, seed=76)
+        got = s.prolong(e)
+        for a, b in ((0, 4), (4, 8), (8, 12), (12, 13)):
+            assert np.array_equal(s.prolong(e[a:b]), got[a:b])
