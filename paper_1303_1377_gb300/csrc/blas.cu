@@ -557,26 +557,6 @@ __device__ __forceinline__ bool last_cta_of_rhs(unsigned* ticket, int r, int cta
     return last;
 }
 
-// Reduce-scatter of NV = 2 KB per-lane FP32 values across a warp (NV a power of two, <= 32): on
-// return v[0] of lane l holds the sum over the 32 lanes of value (l mod NV).  Each halving step
-// sends the half of the live values that the partner lane keeps, so the whole reduction costs
-// NV - 1 shuffles (plus log2(32 / NV) for the lanes beyond NV) instead of 5 NV.
-template <int NV>
-__device__ __forceinline__ void warp_reduce_scatter(float (&v)[NV], int lane) {
-#pragma unroll
-    for (int s = NV / 2; s >= 1; s >>= 1) {
-        const bool upper = lane & s;
-#pragma unroll
-        for (int j = 0; j < s; ++j) {
-            const float send = upper ? v[j] : v[j + s];
-            const float keep = upper ? v[j + s] : v[j];
-            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, s);
-        }
-    }
-#pragma unroll
-    for (int s = NV; s < 32; s <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], s);
-}
-
 template <int KB>
 __global__ void __launch_bounds__(kDotThreads) multidot_f32_kernel(const float4* __restrict__ A, size_t istride4, size_t arstride4, int k,
                                                                    const float4* __restrict__ w, size_t wrstride4, size_t n4, int nrhs,

@@ -89,6 +89,26 @@ __device__ __forceinline__ double arnoldi_column(const KrylovState& s, int r, in
     return __shfl_sync(0xffffffffu, sc, 0);
 }
 
+// Reduce-scatter of NV = 2 KB per-lane FP32 values across a warp (NV a power of two, <= 32): on
+// return v[0] of lane l holds the sum over the 32 lanes of value (l mod NV).  Each halving step
+// sends the half of the live values that the partner lane keeps, so the whole reduction costs
+// NV - 1 shuffles (plus log2(32 / NV) for the lanes beyond NV) instead of 5 NV.
+template <int NV>
+__device__ __forceinline__ void warp_reduce_scatter(float (&v)[NV], int lane) {
+#pragma unroll
+    for (int s = NV / 2; s >= 1; s >>= 1) {
+        const bool upper = lane & s;
+#pragma unroll
+        for (int j = 0; j < s; ++j) {
+            const float send = upper ? v[j] : v[j + s];
+            const float keep = upper ? v[j + s] : v[j];
+            v[j] = keep + __shfl_xor_sync(0xffffffffu, send, s);
+        }
+    }
+#pragma unroll
+    for (int s = NV; s < 32; s <<= 1) v[0] += __shfl_xor_sync(0xffffffffu, v[0], s);
+}
+
 // One Arnoldi step on short FP32 vectors (ortho.cu): V_{k+1} holds A V_k on entry and the next basis vector
 // on exit; the Hessenberg column, the residual estimate and the flags of s are updated.
 bool ortho_step_supported(const cplx<float>* V, size_t bstride, size_t n, int k);

@@ -11,6 +11,7 @@
 
 #include "blas.h"
 #include "kernels.h"
+#include "sum2.cuh"
 
 namespace ddamg {
 
@@ -21,6 +22,7 @@ constexpr int kOrthoCluster = 8, kOrthoThreads = 256, kOrthoWarps = kOrthoThread
 // kernel against four: 320 numbers 32 / 42 us (1 field), 10240 numbers 38 / 48 us (1) and 48 / 61 us (12); at 25920
 // numbers 61 / 62, 72 / 70 (4 fields) and 102 / 111 us (12), where eight CTAs per field begin to be too few.
 constexpr size_t kOrthoMaxSlice = 1024;
+static_assert(kOrthoMaxSlice <= 32 * kLaneWords);
 
 __global__ void __cluster_dims__(kOrthoCluster, 1, 1) __launch_bounds__(kOrthoThreads)
     ortho_step_kernel(KrylovState s, int k, float4* __restrict__ V, size_t bstride4, size_t n4) {
@@ -40,24 +42,18 @@ __global__ void __cluster_dims__(kOrthoCluster, 1, 1) __launch_bounds__(kOrthoTh
     }
     for (int e = tid; e < cnt; e += kOrthoThreads) wsm[e] = w[e];
     __syncthreads();
-    // <V_i, w>: one warp per product, FP32 sums of at most 32 terms a lane, summed over the warp, into FP64
+    // <V_i, w>: one warp per product.  A lane's sums carry their rounding errors along, so that FP32 rounds a term and
+    // five additions over the warp, as in multidot_f32, whatever the length of the slice (30 steps on 10240 numbers: 1.13
+    // -> 1.21 ms; multidot_f32 and the rest as separate kernels 2.17 ms); lanes 0 .. 3 end with the two parts and their
+    // errors, which one FP64 conversion and one addition put together.
     for (int i = wi; i <= k; i += kOrthoWarps) {
-        const float4* a4 = Vr + (size_t)i * bstride4;
-        double re = 0, im = 0;
-        for (int b = lane; b - lane < cnt; b += 32 * 32) {
-            float fr = 0.f, fi = 0.f;
-#pragma unroll 8
-            for (int j = 0; j < 32; ++j) {
-                const int e = b + 32 * j;
-                if (e < cnt) {
-                    const float4 a = a4[e], v = wsm[e];
-                    fr += fmaf(a.x, v.x, a.y * v.y) + fmaf(a.z, v.z, a.w * v.w);
-                    fi += fmaf(a.x, v.y, -a.y * v.x) + fmaf(a.z, v.w, -a.w * v.z);
-                }
-            }
-            re += (double)warp_sum(fr), im += (double)warp_sum(fi);
-        }
-        if (lane == 0) part[2 * i] = re, part[2 * i + 1] = im;
+        Sum2 re, im;
+        lane_dot(Vr + (size_t)i * bstride4, wsm, lane, cnt, re, im);
+        float v[4] = {re.s, im.s, re.e, im.e};
+        warp_reduce_scatter<4>(v, lane);
+        double t = (double)v[0];
+        t += __shfl_down_sync(0xffffffffu, t, 2);
+        if (lane < 2) part[2 * i + lane] = t;
     }
     cl.sync();
     for (int q = tid; q < 2 * (k + 1); q += kOrthoThreads) {
