@@ -178,7 +178,7 @@ __device__ __forceinline__ void stage(__half* x, const cplx<float> (&y)[U], floa
 
 }  // namespace
 
-// grid (blocks of the colour, sets of G groups of four right-hand sides); 32 He threads per group
+// grid: blocks of the colour x sets of G groups of four right-hand sides; 32 He threads per group
 template <int U, int G>
 __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
     ml_sap_tc_kernel(MLView<float> v, const cplx<float>* __restrict__ b, cplx<float>* z, int nrhs, int colour, int mr_steps) {
@@ -186,7 +186,7 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const int He = v.Vb1e, Vb = v.Vb1, NB = v.NB;
     const size_t fs = (size_t)NB * F::NC;
-    const int c2 = colour * (v.NB2 / 2) + blockIdx.x;
+    const int nblk = v.NB2 / 2, c2 = colour * nblk + blockIdx.x % nblk;
     const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31, g = lane >> 2, t = lane & 3;
     const int grp = wid / He, s = wid % He;
     // shared memory: staged vectors of the even sites, the odd sites and each warp's own, [He][SLOT] per
@@ -206,7 +206,7 @@ __global__ void __launch_bounds__(G == 1 ? 512 : 256 * G, 1)
         nbl[q] = v.same[(size_t)d * NB + c] ? v.loc_of[v.nbr1[(size_t)d * NB + c]] : -1;
     }
     __syncthreads();
-    const int r0 = (blockIdx.y * G + grp) * 4;
+    const int r0 = (blockIdx.x / nblk * G + grp) * 4;
     const int nr = nrhs - r0;
     if (nr <= 0) return;  // the barriers below are per group
     auto sync = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(grp + 1), "r"(32 * He) : "memory"); };
@@ -397,7 +397,7 @@ static int launch_ug(const MLView<float>& v, const cplx<float>* b, cplx<float>* 
         return true;
     }();
     (void)attr;
-    const dim3 grid((unsigned)(v.NB2 / 2), (unsigned)ceil_div(nrhs, 4 * G));
+    const unsigned grid = (unsigned)(v.NB2 / 2) * (unsigned)ceil_div(nrhs, 4 * G);
     ml_sap_tc_kernel<U, G><<<grid, 32 * He * G, smem, st>>>(v, b, z, nrhs, colour, mr_steps);
     DD_CHECK_LAUNCH();
     return 0;

@@ -31,7 +31,7 @@ __global__ void __cluster_dims__(kOrthoCluster, 1, 1) __launch_bounds__(kOrthoTh
     __shared__ float2 cs[kOrthoMaxK];
     __shared__ ArnoldiWork aw;
     cg::cluster_group cl = cg::this_cluster();
-    const int r = blockIdx.y, rank = (int)cl.block_rank(), tid = threadIdx.x, wi = tid >> 5, lane = tid & 31, m = s.m;
+    const int r = blockIdx.x / kOrthoCluster, rank = (int)cl.block_rank(), tid = threadIdx.x, wi = tid >> 5, lane = tid & 31, m = s.m;
     const size_t per = (n4 + kOrthoCluster - 1) / kOrthoCluster, e0 = rank * per;
     const int cnt = e0 < n4 ? (int)(n4 - e0 < per ? n4 - e0 : per) : 0;
     const float4* Vr = V + (size_t)r * n4 + e0;              // V_0's slice of this right-hand side
@@ -114,7 +114,7 @@ bool ortho_step_supported(const cplx<float>* V, size_t bstride, size_t n, int k)
 int ortho_step_f32(const KrylovState& s, int k, cplx<float>* V, size_t bstride, size_t n, cudaStream_t st) {
     if (s.m > kOrthoMaxK || k >= s.m) return DDAMG_ERR_INVALID_ARG;
     const size_t n4 = n / 2, per = (n4 + kOrthoCluster - 1) / kOrthoCluster;
-    ortho_step_kernel<<<dim3(kOrthoCluster, s.nrhs), kOrthoThreads, per * sizeof(float4), st>>>(s, k, reinterpret_cast<float4*>(V), bstride / 2, n4);
+    ortho_step_kernel<<<(unsigned)kOrthoCluster * (unsigned)s.nrhs, kOrthoThreads, per * sizeof(float4), st>>>(s, k, reinterpret_cast<float4*>(V), bstride / 2, n4);
     DD_CHECK_LAUNCH();
     return 0;
 }

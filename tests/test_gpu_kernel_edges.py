@@ -330,3 +330,21 @@ def test_half_prolongation_gives_the_same_bits_by_either_route():
         got = s.prolong(e)
         for a, b in ((0, 4), (4, 8), (8, 12), (12, 13)):
             assert np.array_equal(s.prolong(e[a:b]), got[a:b])
+
+
+@pytest.mark.parametrize("prec,n_vec", [("SINGLE", 1), ("HALF", 24)])
+def test_level1_calls_with_more_fields_than_a_grid_row(prec, n_vec):
+    """262145 fields, more groups of four than grid.y may have: the last fields come out as in a batch of their own."""
+    import torch
+
+    from paper_1303_1377_gb300 import ddamg
+
+    s, _ = _solver((4, 4, 4, 8), n_vec=n_vec, block=(2, 2, 2, 2), precision=getattr(ddamg, "PREC_" + prec))
+    with s:
+        s.setup_from_vectors(synth.random_test_vectors((4, 4, 4, 8), n_vec, seed=1))
+        s.ml_build(synth.gaussian_coarse(32, 2 * n_vec, 1, seed=2), ddamg.ml_default_params(n_vec1=1, block1=(1, 1, 1, 2)))
+        x = torch.zeros((262145, 32, 2 * n_vec), dtype=torch.complex128, device="cuda")
+        x[-3:] = torch.from_numpy(synth.gaussian_coarse(32, 2 * n_vec, 3, seed=3))
+        last = x[-3:].contiguous()
+        assert torch.equal(s.ml_restrict1(x)[-3:], s.ml_restrict1(last))
+        assert torch.equal(s.ml_apply_sap1(x, 1)[-3:], s.ml_apply_sap1(last, 1))
