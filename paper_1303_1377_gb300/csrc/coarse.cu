@@ -173,12 +173,7 @@ static int launch_stencil_threads(const CoarseOp<S>& op, int site_begin, int nsi
     size_t stage = (size_t)9 * op.nc * NRP * sizeof(cplx<T>);
     size_t reduce = (size_t)(KG + 1) * op.nc * NRP * sizeof(cplx<T>);
     size_t smem = stage > reduce ? stage : reduce;
-    // set once per kernel instance (a function-local static initialiser is thread safe)
-    static const bool attr = [] {
-        cudaFuncSetAttribute(coarse_stencil_kernel<T, S, NRP, WIDE, UNR>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        return true;
-    }();
-    (void)attr;
+    DD_CUDA((allow_smem<coarse_stencil_kernel<T, S, NRP, WIDE, UNR>>(200 * 1024)));
     coarse_stencil_kernel<T, S, NRP, WIDE, UNR><<<nsites, nt, smem, st>>>(op, site_begin, xin, xself, self_mode, hop_sign, apply_inv, out, nrhs);
     DD_CHECK_LAUNCH();
     return 0;

@@ -346,13 +346,8 @@ template <int NRP>
 static int launch_tc_nrp(const CoarseTC& op, int site_begin, int nsites, CVecT<float> xin, CVecT<float> xself, int self_mode,
                          float hop_sign, int apply_inv, CVecT<float> out, int nrhs, cudaStream_t st) {
     const size_t smem = tc_smem(op, NRP, self_mode, hop_sign, apply_inv);
-    // set once per kernel instance (a function-local static initialiser is thread safe)
-    static const bool attr = [] {
-        cudaFuncSetAttribute(coarse_tc_kernel<NRP, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax);
-        if constexpr (NRP <= 12) cudaFuncSetAttribute(coarse_tc_kernel<NRP, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax);
-        return true;
-    }();
-    (void)attr;
+    DD_CUDA((allow_smem<coarse_tc_kernel<NRP, false>>((int)kTcSmemMax)));
+    if constexpr (NRP <= 12) DD_CUDA((allow_smem<coarse_tc_kernel<NRP, true>>((int)kTcSmemMax)));
     if constexpr (NRP <= 12) {  // split staging: at most 12 right-hand sides per launch (no register spills)
         if (op.split) {
             coarse_tc_kernel<NRP, true><<<nsites, 64 * op.Mt, smem, st>>>(op, site_begin, xin, xself, self_mode, hop_sign, apply_inv, out,

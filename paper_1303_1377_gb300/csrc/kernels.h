@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 
 #include "common.cuh"
+#include "device_once.h"
 #include "../../include/ddamg.h"
 
 namespace ddamg {

@@ -265,12 +265,8 @@ bool ml_sap_fused_supported(const MLView<float>& v) {
 int launch_ml_sap_fused(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps,
                         cudaStream_t st) {
     const size_t smem = ml_sap_fused_smem(v);
-    static const bool attr = [] {
-        cudaFuncSetAttribute(ml_sap_fused_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        cudaFuncSetAttribute(ml_sap_fused_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-        return true;
-    }();
-    (void)attr;
+    DD_CUDA(allow_smem<ml_sap_fused_kernel<false>>(227 * 1024));
+    DD_CUDA(allow_smem<ml_sap_fused_kernel<true>>(227 * 1024));
     const int threads = ((kG * v.Vb1e * v.nc + 31) / 32) * 32;
     const dim3 grid((unsigned)(v.NB2 / 2), (unsigned)((nrhs + kR - 1) / kR));
     if (v.B1h && v.Dinv1h)

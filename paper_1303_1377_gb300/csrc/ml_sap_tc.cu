@@ -391,12 +391,7 @@ static int launch_ug(const MLView<float>& v, const cplx<float>* b, cplx<float>* 
     const int He = v.Vb1e;
     const size_t smem = (size_t)3 * G * He * F::SLOT * sizeof(__half) + (size_t)G * He * 2 * U * 32 * sizeof(cplx<float>) +
                         (size_t)G * He * 12 * sizeof(float) + (size_t)v.Vb1 * 9 * sizeof(int);
-    // set once per kernel instance (a function-local static initialiser is thread safe)
-    static const bool attr = [] {
-        cudaFuncSetAttribute(ml_sap_tc_kernel<U, G>, cudaFuncAttributeMaxDynamicSharedMemorySize, 200 * 1024);
-        return true;
-    }();
-    (void)attr;
+    DD_CUDA((allow_smem<ml_sap_tc_kernel<U, G>>(200 * 1024)));
     const unsigned grid = (unsigned)(v.NB2 / 2) * (unsigned)ceil_div(nrhs, 4 * G);
     ml_sap_tc_kernel<U, G><<<grid, 32 * He * G, smem, st>>>(v, b, z, nrhs, colour, mr_steps);
     DD_CHECK_LAUNCH();

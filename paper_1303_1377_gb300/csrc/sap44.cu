@@ -472,12 +472,7 @@ int launch_sap44(const Geom& g, const OpT& op, const cplx<float>* b, cplx<float>
         return 0;
     }
     const size_t smem = 24 * 128 * sizeof(float4) + 12 * sizeof(float2);
-    // set once per kernel instance (a function-local static initialiser is thread safe)
-    static const bool attr = [] {
-        cudaFuncSetAttribute(sap44_kernel<OpT>, cudaFuncAttributeMaxDynamicSharedMemorySize, 100 * 1024);
-        return true;
-    }();
-    (void)attr;
+    DD_CUDA(allow_smem<sap44_kernel<OpT>>(100 * 1024));
     const int npairs = (nrhs + 1) / 2;
     sap44_kernel<OpT><<<(unsigned)(g.NB / 2) * (unsigned)npairs, 128, smem, st>>>(g, op, b, z, colour, nrhs, mr_steps, npairs);
     DD_CHECK_LAUNCH();

@@ -430,9 +430,7 @@ static int build_geometry(ddamg_handle* h) {
 }
 
 // gamma_mu gamma_nu (mu < nu) chiral blocks, from the gamma matrices of Sec. 2.2
-static int upload_gammas() {
-    static bool done = false;
-    if (done) return 0;
+static int upload_gammas_here() {
     typedef std::array<std::array<std::array<double, 2>, 4>, 4> G4;
     G4 gm[4];
     for (auto& g : gm)
@@ -468,9 +466,14 @@ static int upload_gammas() {
                         gg[plane][hh][s][t][1] = prod[2 * hh + s][2 * hh + t][1];
                     }
         }
-    DD_TRY(upload_gamma_products(&gg[0][0][0][0][0]));
-    done = true;
-    return 0;
+    return upload_gamma_products(&gg[0][0][0][0][0]);
+}
+static int upload_gammas() {
+    static DeviceOnce once;
+    const int rc = once(upload_gammas_here);
+    if (rc <= 0) return rc;
+    set_error(std::string("cudaGetDevice: ") + cudaGetErrorString((cudaError_t)rc));
+    return DDAMG_ERR_CUDA;
 }
 
 static bool is_device_ptr(const void* p) {
