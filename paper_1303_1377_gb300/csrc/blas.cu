@@ -146,7 +146,8 @@ int convert(const Ti* in, To* out, size_t n, cudaStream_t st) {
 
 // ABI lexicographic field [nrhs][V][ncomp] <-> internal [nrhs][ncomp][V];  lex_of[i] = lexicographic site of internal i
 // MAX: also rmax[r] = bits of max |Re|, |Im| of right-hand side r as stored (non-negative floats order like their
-// bits).  V is a multiple of 256, so a CTA's 256 sites belong to one right-hand side.
+// bits).  V is a multiple of 256 (even block extents, an even number of blocks in every direction), so a CTA's 256
+// sites belong to one right-hand side.
 template <typename To, typename Ti, bool MAX>
 __global__ void __launch_bounds__(256) to_internal_kernel(const cplx<Ti>* __restrict__ in, cplx<To>* __restrict__ out,
                                                           const int* __restrict__ lex_of, int V, int ncomp, int nrhs, int* __restrict__ rmax) {
@@ -215,7 +216,6 @@ int to_internal(const cplx<Ti>* in, cplx<To>* out, const int* lex_of, int V, int
     return 0;
 }
 int to_internal_max(const cplx<double>* in, cplx<float>* out, const int* lex_of, int V, int ncomp, int nrhs, int* rmax, cudaStream_t st) {
-    if (V % 256) return DDAMG_ERR_INVALID_ARG;
     int blocks = ceil_div((long long)V * nrhs, 256);
     if (blocks > 152 * 32) blocks = 152 * 32;
     DD_CUDA(cudaMemsetAsync(rmax, 0, sizeof(int) * nrhs, st));

@@ -154,7 +154,7 @@ template <typename To, typename Ti>
 int convert(const Ti* in, To* out, size_t n, cudaStream_t st);
 template <typename To, typename Ti>
 int to_internal(const cplx<Ti>* in, cplx<To>* out, const int* lex_of, int V, int ncomp, int nrhs, cudaStream_t st);
-// to_internal<float, double> that also leaves the bits of max |Re|, |Im| of each field in rmax (V % 256 == 0)
+// to_internal<float, double> that also leaves the bits of max |Re|, |Im| of each field in rmax
 int to_internal_max(const cplx<double>* in, cplx<float>* out, const int* lex_of, int V, int ncomp, int nrhs, int* rmax, cudaStream_t st);
 template <typename To, typename Ti>
 int from_internal(const cplx<Ti>* in, cplx<To>* out, const int* lex_of, int V, int ncomp, int nrhs, cudaStream_t st);

@@ -79,16 +79,12 @@ __device__ __noinline__ void dw_hop_rt(cdw (&acc)[12], const cplx<float>* __rest
 
 }  // namespace
 
-// thread (x, y): site blockIdx.x * 32 + x, right-hand side blockIdx.y * blockDim.y + y (the warps of
-// a CTA share the double-word links and site terms of 32 sites through L1)
+// one right-hand side: a thread per site, one warp per CTA
 template <bool OUT_DW>
 __global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __restrict__ U, const float2* __restrict__ clov,
-                                                        const cplx<float>* __restrict__ in, void* __restrict__ outp, int nrhs) {
-    const int r = blockIdx.y * blockDim.y + threadIdx.y;
+                                                        const cplx<float>* __restrict__ inr, void* __restrict__ outp) {
     const int i = blockIdx.x * 32 + threadIdx.x;
-    if (i >= g.V || r >= nrhs) return;
-    const size_t off = (size_t)r * 12 * g.V;
-    const cplx<float>* inr = in + off;
+    if (i >= g.V) return;
     cdw acc[12];
 #pragma unroll
     for (int k = 0; k < 12; ++k) acc[k] = cdw_zero();
@@ -140,7 +136,7 @@ __global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __
         }
     }
     if (OUT_DW) {
-        float4* o = reinterpret_cast<float4*>(outp) + off;
+        float4* o = reinterpret_cast<float4*>(outp);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             dw re = dw_norm(dw_add(y[k].re, {-0.5f * acc[k].re.h, -0.5f * acc[k].re.l}));
@@ -148,7 +144,7 @@ __global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __
             o[(size_t)k * g.V + i] = make_float4(re.h, re.l, im.h, im.l);
         }
     } else {
-        cplx<double>* o = reinterpret_cast<cplx<double>*>(outp) + off;
+        cplx<double>* o = reinterpret_cast<cplx<double>*>(outp);
 #pragma unroll
         for (int k = 0; k < 12; ++k) {
             double re = (double)y[k].re.h + (double)y[k].re.l - 0.5 * ((double)acc[k].re.h + (double)acc[k].re.l);
@@ -376,9 +372,9 @@ int launch_dslash_dw(const Geom& g, const float4* U, const float2* clov, const c
         DD_CHECK_LAUNCH();
         return 0;
     }
-    const dim3 grid((unsigned)ceil_div(g.V, 32), 1), block(32, 1);
-    if (out_dw) dslash_dw_kernel<true><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
-    else dslash_dw_kernel<false><<<grid, block, 0, st>>>(g, U, clov, in, out, nrhs);
+    const unsigned grid = (unsigned)ceil_div(g.V, 32);
+    if (out_dw) dslash_dw_kernel<true><<<grid, 32, 0, st>>>(g, U, clov, in, out);
+    else dslash_dw_kernel<false><<<grid, 32, 0, st>>>(g, U, clov, in, out);
     DD_CHECK_LAUNCH();
     return 0;
 }

@@ -31,14 +31,14 @@ __device__ __forceinline__ void hop_pair_nb(const UT& U, const cplx<Ts>* __restr
     hop_acc<MU, false>(acc, pn, W);
 }
 
-// out = D in (RESID: out = b - D in) on 4^4 blocks, FP64 and single FP32 fields (two and more FP32
-// fields: dslash44.cu).  CTA = 32 sites of one block x ry right-hand sides (one warp per right-hand
+// out = D in (RESID: out = b - D in) on 4^4 blocks, FP64 fields and single FP32 fields (two and more FP32
+// fields: dslash44.cu).  CTA = 32 sites of one block x ry <= 4 right-hand sides (one warp per right-hand
 // side, sharing the links and site terms through L1).  The CTAs walk
 // the blocks in lexicographic block order, red and black interleaved, so that a block and its
 // neighbours in three of the four directions are read close together in time and the neighbours'
-// spinors are still in L2.
+// spinors are still in L2.  (FP32: 80 registers, 24 warps per SM.)
 template <typename T, typename Ts, bool RESID>
-__global__ void __launch_bounds__(sizeof(T) == 4 ? 384 : 128, sizeof(T) == 4 ? 2 : 1)
+__global__ void __launch_bounds__(128, sizeof(T) == 4 ? 6 : 1)
     dslash44_kernel(Geom g, FineOp<T> op, const int* __restrict__ blex, const cplx<Ts>* __restrict__ in, const cplx<T>* __restrict__ b,
                     cplx<T>* __restrict__ out, int nrhs, const int* __restrict__ lex) {
     const int r = blockIdx.y * blockDim.y + threadIdx.y;
@@ -131,8 +131,8 @@ __global__ void __launch_bounds__(sizeof(T) == 4 ? 384 : 128, sizeof(T) == 4 ? 2
 template <typename T, typename Ts>
 int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const cplx<T>* b, cplx<T>* out, int nrhs, cudaStream_t st,
                   const int* lex) {
-    const int ry = std::min(nrhs, sizeof(T) == 4 ? 12 : 4);  // right-hand sides per CTA
     if (g.blk44 && g.blex) {
+        const int ry = std::min(nrhs, 4);  // right-hand sides per CTA
         const dim3 grid((unsigned)g.NB * 8, (unsigned)ceil_div(nrhs, ry)), block(32, ry);
         if (b)
             dslash44_kernel<T, Ts, true><<<grid, block, 0, st>>>(g, op, g.blex, in, b, out, nrhs, lex);
@@ -142,6 +142,7 @@ int launch_dslash(const Geom& g, const FineOp<T>& op, const cplx<Ts>* in, const 
         return 0;
     }
     if (lex) return DDAMG_ERR_INVALID_ARG;
+    const int ry = std::min(nrhs, sizeof(T) == 4 ? 12 : 4);
     const dim3 grid((unsigned)ceil_div(g.V, 32), (unsigned)ceil_div(nrhs, ry)), block(32, ry);
     if (b)
         dslash_kernel<T, Ts, true><<<grid, block, 0, st>>>(g, op, in, b, out, nrhs);

@@ -2117,7 +2117,7 @@ static int restrict_T(ddamg_handle* h, const double* in, double* out, int n_rhs)
     cplx<T>* o = a + fld * n_rhs;
     bool have_max = false;
     if constexpr (std::is_same<T, float>::value) {
-        if (h->half() && restrict_tc_supported(h->g, h->N) && h->V % 256 == 0) {
+        if (h->half() && restrict_tc_supported(h->g, h->N)) {
             // the FP16 restriction scales by the fields' maxima: found while the fields are brought in
             const void* dv;
             DD_TRY(h->ws_rmax.ensure(sizeof(int) * n_rhs));
