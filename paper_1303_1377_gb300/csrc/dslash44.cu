@@ -2,11 +2,9 @@
 //
 // Bound by the latency of the neighbours' spinors.  A CTA of 128 threads covers half a block (64 sites of
 // either parity) and one pair of right-hand sides: 128 registers leave 16 warps on an SM, and most in-block
-// neighbours are sites of the same CTA, so their spinors hit L1.  12 fields of 32^4, the call: 1785 us; a CTA of
-// 32 sites and up to six pairs (168 registers, 12 warps, operator shared through L1) 1980 us, whole blocks
-// (256 threads) 1806 us, quarter blocks 1870 us; 226 registers, two CTAs per SM, 1972 us; 12 fields of 24^4
-// 600 against 648 us, two of 16^3 x 32 92 against 90 us.  One right-hand side per thread (24 warps, 80
-// registers) took 1646 us for the kernel alone against 1290 us in the six-pair form.
+// neighbours are sites of the same CTA, so their spinors hit L1.  The call against one right-hand side per thread
+// (24 warps, 80 registers): 12 fields of 32^4 3669 -> 1785 us, two fields of 8^4 (32 CTAs) 53 -> 43 us, of 16^4 79 ->
+// 55 us, three of 24x16^3 122 -> 87 us.
 #include <type_traits>
 
 #include "ops44.cuh"

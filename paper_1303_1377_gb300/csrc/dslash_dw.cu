@@ -161,11 +161,9 @@ __global__ void __launch_bounds__(128) dslash_dw_kernel(Geom g, const float4* __
 // Two threads share a site: thread s takes row s of the projected half spinors in the hops (the upper row s and
 // one lower row out) and chirality half s of the site term; their parts meet by shuffles after the last hop.
 // Bound by the latency of its chains (a double-word multiply-add is 12 packed instructions of two cycles) at 12
-// warps per SM (168 registers); one thread per site held 24 accumulators and ran 8 warps of 254 registers: 12
-// fields of 24^4, the call, 3600 -> 3280 us (3000 with the pairs dealt out as in launch_dslash_dw), five of
-// 8x16x8x24 184 -> 168 us, two of 16^3 x 32 271 -> 278 us; error against 64 bits 5.8e-15 both.  Before the pairs
-// were dealt out: the accumulators parked in shared memory during the site term 3410 us; four CTAs per SM (spills)
-// 3530 us; the site term added straight onto -acc / 2 2910 us, but the error rises to 7.5e-15.
+// warps per SM (168 registers; one thread per site held 24 accumulators, 254 registers, 8 warps).  The call against
+// one right-hand side per thread: 12 fields of 24^4 4680 -> 3000 us, two of 8^4 90 -> 62 us, of 16^4 208 -> 168 us;
+// error against 64 bits 5.8e-15 both.  (The site term added straight onto -acc / 2 is quicker but errs by 7.5e-15.)
 // The loop over the eight directions is rolled (one hop is about 10 KB of code) with the spin structure as
 // run-time selects and sign flips on the integer pipe.  FP64 instructions issue at 1/64 of the FP32 rate,
 // conversions included: y - acc / 2 is summed in FP32 words and takes one FP64 addition a number (formed in

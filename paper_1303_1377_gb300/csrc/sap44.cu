@@ -8,12 +8,9 @@
 // terms that every MR step reads again.
 //
 // What bounds it: the packed multiply-adds (two cycles each) hold the FMA pipe about 60% busy in the MR
-// steps; the residual at the start waits on its neighbours' spinors.  12 fields on 24^4, one colour,
-// FP16 operator: 740 us (29 TFLOP/s) against 1347 us for one right-hand side per thread, four per CTA
-// (512 threads, 128 registers); FP32 operator 740 against 1399 us.  Few blocks, or one field: sap44_one_kernel below.  Tried
-// and slower (same case): four right-hand sides per CTA 778 us, six 806 us; x_o in shared memory
-// (+12%); the links in shared memory as FP32 (+5%); two threads per site split by spin 781 us; own z
-// and the faces staged through shared memory (+15%).
+// steps; the residual at the start waits on its neighbours' spinors.  12 fields on 24^4, one colour: 740 us
+// (29 TFLOP/s) with either operator; one right-hand side per thread, four per CTA (512 threads, 128 registers), took
+// 1347 us (FP16) and 1399 us (FP32).  One field, or few blocks: sap44_one_kernel, by the rule in launch_sap44.
 #include <type_traits>
 
 #include "ops44.cuh"
