@@ -43,9 +43,9 @@ __global__ void __cluster_dims__(kOrthoCluster, 1, 1) __launch_bounds__(kOrthoTh
     for (int e = tid; e < cnt; e += kOrthoThreads) wsm[e] = w[e];
     __syncthreads();
     // <V_i, w>: one warp per product.  A lane's sums carry their rounding errors along, so that FP32 rounds a term and
-    // five additions over the warp, as in multidot_f32, whatever the length of the slice (30 steps on 10240 numbers: 1.13
-    // -> 1.21 ms; multidot_f32 and the rest as separate kernels 2.17 ms); lanes 0 .. 3 end with the two parts and their
-    // errors, which one FP64 conversion and one addition put together.
+    // five additions over the warp, as in multidot_f32, whatever the length of the slice (30 steps on 10240 numbers: 1.09
+    // ms, with plain sums word by word 1.12 ms; multidot_f32 and the rest as separate kernels 2.17 ms); lanes 0 .. 3 end
+    // with the two parts and their errors, which one FP64 conversion and one addition put together.
     for (int i = wi; i <= k; i += kOrthoWarps) {
         Sum2 re, im;
         lane_dot(Vr + (size_t)i * bstride4, wsm, lane, cnt, re, im);

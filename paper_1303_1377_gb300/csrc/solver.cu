@@ -244,7 +244,7 @@ struct ddamg_handle {
     double *clov64 = nullptr, *clovinv64 = nullptr;
     cplx<float>* U32 = nullptr;
     float *clov32 = nullptr, *clovinv32 = nullptr;
-    float4 *Uaos = nullptr, *clov_aos = nullptr, *clovinv_aos = nullptr;  // per-site FP32 copies for the SAP
+    float4 *Uaos = nullptr, *clov_aos = nullptr, *clovinv_aos = nullptr;  // per-site FP32 copies (4^4 blocks: per block)
     uint4 *Uaos16 = nullptr, *clov_aos16 = nullptr, *clovinv_aos16 = nullptr;  // half mode: FP16 per-site copies
     float4* Udw = nullptr;    // links as double-word FP32 pairs (FGMRES matvec on FP32 inputs)
     float2* clovdw = nullptr;  // site terms as double-word pairs

@@ -18,16 +18,25 @@ struct Sum2 {
 };
 
 // one lane's part of <a, w>, two complex numbers a float4: words first, first + 32, ... below cnt, at most
-// kLaneWords of them
+// kLaneWords of them; first < 32.  Eight words at a time without branches (zeros past the end), so that their loads
+// and the error terms of their additions overlap.
 constexpr int kLaneWords = 32;
 __host__ __device__ __forceinline__ void lane_dot(const float4* a4, const float4* w4, int first, int cnt, Sum2& re, Sum2& im) {
-#pragma unroll 8
-    for (int j = 0; j < kLaneWords; ++j) {
-        const int e = first + 32 * j;
-        if (e < cnt) {
-            const float4 a = a4[e], v = w4[e];
-            re.add(fmaf(a.x, v.x, a.y * v.y) + fmaf(a.z, v.z, a.w * v.w));
-            im.add(fmaf(a.x, v.y, -a.y * v.x) + fmaf(a.z, v.w, -a.w * v.z));
+    constexpr int B = 8;
+#pragma unroll 1
+    for (int j = 0; j < 32 * kLaneWords && j < cnt; j += 32 * B) {
+        float4 a[B], v[B];
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+            const int e = j + 32 * q + first;
+            const bool on = e < cnt;
+            a[q] = on ? a4[e] : float4{0.f, 0.f, 0.f, 0.f};
+            v[q] = on ? w4[e] : float4{0.f, 0.f, 0.f, 0.f};
+        }
+#pragma unroll
+        for (int q = 0; q < B; ++q) {
+            re.add(fmaf(a[q].x, v[q].x, a[q].y * v[q].y) + fmaf(a[q].z, v[q].z, a[q].w * v[q].w));
+            im.add(fmaf(a[q].x, v[q].y, -a[q].y * v[q].x) + fmaf(a[q].z, v[q].w, -a[q].w * v[q].z));
         }
     }
 }
