@@ -346,7 +346,8 @@ void ddamg_debug_fail_allocs(int n);
  *   the level-1 V-cycle (inner = 0), or one level-1 V-cycle (inner = 1).
  * P_1, D_2 and its inverses are built in FP64; the level-1 and level-2 solves run in the handle's
  * V-cycle precision (FP64 on DOUBLE handles, FP32 on SINGLE and HALF handles, with FP32 copies of
- * D_1, P_1, D_2 and the inverses).  HALF handles also keep FP16 copies: the level-1 SAP reads D_1 and
+ * D_1, P_1, D_2 and the inverses).  HALF handles also keep FP16 copies: where a block has at most 341
+ * pairs (even site, component), as with 2^4 blocks up to n_vec = 20, the level-1 SAP reads D_1 and
  * its even inverses in FP16 (the vectors enter in FP32, or as FP16 hi + lo pairs on the tensor cores,
  * scaled by a power of two per block and field so that a field may have any size that FP32 holds,
  * with FP32 accumulation), and the coarsest level's GMRES and ddamg_ml_apply_D2

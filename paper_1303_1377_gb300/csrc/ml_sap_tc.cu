@@ -399,10 +399,10 @@ static int launch_ug(const MLView<float>& v, const cplx<float>* b, cplx<float>* 
 }
 template <int U>
 static int launch_u(const MLView<float>& v, const cplx<float>* b, cplx<float>* z, int nrhs, int colour, int mr_steps, cudaStream_t st) {
-    // Three groups per CTA read each matrix block once from L2 (12 fields, 128 blocks of nc = 40: 150 us a
-    // colour against 169 us with one group per CTA); one group per CTA spreads few blocks over more SMs
-    // (16 blocks: 62 against about 134 us).  The line is one CTA per SM at one group each.  At nc = 48 the 80
-    // registers of the wide form spill (blocks of 8 sites, the call: 826 us with one group, 996 us with three).
+    // Three groups per CTA read each matrix block once from L2 (12 fields, 128 blocks of nc = 40, the call: 641 us
+    // against 695 us with one group per CTA); one group per CTA spreads few blocks over more SMs (16 blocks, a
+    // colour: 62 against about 134 us).  The line is one CTA per SM at one group each.  At nc = 48 the 80 registers
+    // of the wide form spill (blocks of 8 sites, the call: 826 us with one group, 996 us with three).
     const bool wide = v.Vb1e <= 8 && nrhs > 4 && (long long)(v.NB2 / 2) * ceil_div(nrhs, 4) > 152;
     if constexpr (U < 6)
         if (wide) return launch_ug<U, 3>(v, b, z, nrhs, colour, mr_steps, st);
